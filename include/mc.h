@@ -74,7 +74,11 @@ typedef struct mc_options {
     int32_t pr_level;        /* Padberg-Rinaldi tests 1..pr_level, 0 = off;
                                 PR1/PR2 run every round, PR3/PR4 in rounds whose
                                 scans unite < n/4 vertices; default 4           */
-    int32_t scans_per_round; /* concurrent CAPFOREST warps, 0 = auto           */
+    int32_t scans_per_round; /* concurrent CAPFOREST warps, 0 = auto.  Asking for
+                                something of the scans (this, region_budget,
+                                visits, MC_PQ_FIFO) has them run every round;
+                                else graphs that are not clustered take forest
+                                packing first                                  */
     int32_t region_budget;   /* max vertices touched by one scan, 0 = auto
                                 (192; 320 on graphs with >= 48 arcs/vertex;
                                 64 on graphs below 2^17 vertices)            */
@@ -120,7 +124,8 @@ typedef struct mc_stats {
                                 the clustered remainder, whose phases are also
                                 counted below                                  */
     double ms_pr;            /* Padberg-Rinaldi tests                           */
-    double ms_capforest;     /* CAPFOREST scans (parallel + fallback)           */
+    double ms_capforest;     /* connectivity certificates: forest packing,
+                                CAPFOREST scans (parallel + fallback)           */
     double ms_contract;      /* union-find flatten, relabel, sort, rebuild      */
     int64_t bytes_alg;       /* algorithmic bytes the method had to move        */
     int64_t scanned_arcs;    /* arcs read by CAPFOREST scans                    */

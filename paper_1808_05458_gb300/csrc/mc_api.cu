@@ -1,8 +1,10 @@
 // mc_api.cu -- the C ABI (include/mc.h) and the host driver of Alg. 2.
 //
 // Driver per round on the current graph G_C (Alg. 2, Sec. 3.3):
-//   union-find reset -> Padberg-Rinaldi tests -> concurrent capped CAPFOREST
-//   (Alg. 1) -> if nothing was united: one full CAPFOREST scan (Alg. 3) ->
+//   union-find reset -> Padberg-Rinaldi tests -> forest packing (mc_forest.cu)
+//   or, on clustered graphs and where it unites little, concurrent capped
+//   CAPFOREST (Alg. 1) -> if nothing was united: one full CAPFOREST scan
+//   (Alg. 3) ->
 //   contraction (Sec. 3.2) -> lambda-hat = min(lambda-hat, delta(G_C)).
 // Every improvement of lambda-hat snapshots its side as a bitmap over the
 // original vertices (Sec. 3.3): a scan's prefix for an alpha cut, the
@@ -29,6 +31,7 @@ struct mc_graph {
     int argmin0 = 0;
     i64 wmax0 = 0;          // largest arc weight of G0
     i64 two_arc_rows0 = 0;  // rows of G0 with exactly two arcs
+    bool clustered = false; // most wedges of G0 are closed (k_graph_stats)
     bool device_ptrs = false;
     bool complete = false;  // every buffer allocated and the input built
     std::vector<cudaEvent_t> events;  // phase-clock events, reused across calls
@@ -287,6 +290,7 @@ int create_impl(int32_t n, const int32_t *row_ptr, const int32_t *col, const int
         g->argmin0 = g->w.h_st->argmin;
         g->wmax0 = g->w.h_st->count;
         g->two_arc_rows0 = g->w.h_st->count2;
+        g->clustered = 2 * g->w.h_st->closed > g->w.h_st->wedges;
         if (g->delta0 >= (1LL << 62)) rc = MC_EOVERFLOW;
     }
     if (rc != MC_OK) {
@@ -459,6 +463,10 @@ int solve_impl(mc_graph *g, const mc_options &o, cudaStream_t s, SolveOut &out) 
     int rounds = 0, fallbacks = 0;
     const int tail_n = o.tail_vertices == 0 ? 256 : (o.tail_vertices > 4096 ? 4096 : o.tail_vertices);
     const bool verbose = getenv("MC_VERBOSE") != nullptr;
+// forest packing in place of the concurrent scans, unless the options ask
+    // for something of the scans (mc_forest.cu on which graphs gain by it)
+    const bool pack_forests = !g->clustered && o.pq_order != MC_PQ_FIFO && o.visits <= 1 && o.region_budget <= 0 &&
+                              o.scans_per_round <= 0;
 
     // Alg. 2's loop from `cur`, contracting into the free buffer of Ga / Gb;
     // lowers lam and records sides through w.orig
@@ -544,7 +552,22 @@ int solve_impl(mc_graph *g, const mc_options &o, cudaStream_t s, SolveOut &out) 
             return MC_OK;
         };
         i64 unions = 0;
-        MC_TRY(scan_round(cfg.budget, &unions));
+        // forest packing; a round of it that unites less than an eighth of the
+        // vertices has the scans try as well
+        bool packed = false;
+        if (pack_forests && forest_fits(cur, w, thr)) {
+            MC_TRY(forest_round(cur, w, thr, s));
+            MC_TRY(status_read(w, s));
+            unions = w.h_st->unions;
+            packed = unions * 8 >= cur.n;
+            // heads of the rows, and each parent written once and read twice
+            bytes += (i64)cur.n * thr * 20 + (i64)cur.n * 16;
+            if (verbose)
+                fprintf(stderr, "[mc] round %d n=%d arcs=%lld lam=%lld forests: unions=%lld\n", rounds, cur.n,
+                        (long long)cur.arcs, (long long)thr, (long long)unions);
+        }
+        const bool one_block = packed && unions * 2 >= cur.n;
+        if (!packed) MC_TRY(scan_round(cfg.budget, &unions));
         ph.mark(&S.ms_capforest);
         // a poor round: the triangle tests PR3/PR4 add their unions, on the
         // edges whose shorter row has at most 16 arcs (their work grows with
@@ -597,7 +620,7 @@ int solve_impl(mc_graph *g, const mc_options &o, cudaStream_t s, SolveOut &out) 
         MC_TRY(contract_graph(cur, *nxt, w, lam, true, 0, s, [&]() -> int {
             MC_TRY(orig_update(w, n0, s));
             return min_degree(*nxt, w, s);
-        }));
+        }, one_block));
         if (w.h_st->err & kErrOverflow) return MC_EOVERFLOW;
         if (w.h_st->err & kErrNoProgress) return MC_EINTERNAL;
         bytes += cur.arcs * 20 + w.last_emitted * 12 + (i64)cur.n * 16 + (i64)n0 * 8;

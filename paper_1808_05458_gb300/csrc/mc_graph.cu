@@ -245,6 +245,86 @@ k_emit(const int *__restrict__ src, const int2 *__restrict__ adj, i64 arcs, cons
     }
 }
 
+// The same arcs read from the rows outside one block that holds most of the
+// vertices: an arc from that block is the mirror of one of theirs.  A row's
+// weight into the block is added up (saturated like the rest) and emitted once
+// in both directions.  A warp a row; what a warp finds waits in shared memory
+// and goes out 64 or more at a time, one atomic each.  Against reading every
+// arc (10-core of an R-MAT graph, 29 M arcs, one block of all but a few
+// vertices): 105 -> 8 us.
+constexpr int kOutBuf = 128;
+
+__global__ void __launch_bounds__(kThreads)
+k_emit_outside(const DevGraph g, const int *__restrict__ lab, const int *giant, const int *d_nc, i64 clamp, int wb,
+               u64 *__restrict__ keys, int *__restrict__ vals, u64 *counter) {
+    __shared__ u64 bkey[kThreads / 32][kOutBuf];
+    __shared__ int bval[kThreads / 32][kOutBuf];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const u64 nc = (u64)*d_nc;
+    const int big = lab[*giant];
+    const long long cap = clamp < (i64)kInt32Max ? clamp : (i64)kInt32Max;
+    int held = 0;
+    auto flush = [&]() {
+        __syncwarp();
+        u64 base = 0;
+        if (lane == 0) base = atomicAdd(counter, (u64)held);
+        base = __shfl_sync(0xffffffffu, base, 0);
+        for (int i = lane; i < held; i += 32) {
+            if (wb) {
+                keys[base + i] = (bkey[wid][i] << wb) | (u64)(unsigned)bval[wid][i];
+            } else {
+                keys[base + i] = bkey[wid][i];
+                vals[base + i] = bval[wid][i];
+            }
+        }
+        held = 0;
+        __syncwarp();
+    };
+    const int nw = (gridDim.x * blockDim.x) >> 5;
+    for (int v0 = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32; v0 < g.n; v0 += nw * 32) {
+        const int vl = v0 + lane;
+        const int al = vl < g.n ? lab[vl] : big;
+        unsigned todo = __ballot_sync(0xffffffffu, al != big);
+        while (todo) {
+            const int l = __ffs(todo) - 1;
+            todo &= todo - 1;
+            const int u = v0 + l, a = __shfl_sync(0xffffffffu, al, l);
+            const int a1 = g.rp[u + 1];
+            long long into = 0;
+            for (int i0 = g.rp[u]; i0 < a1; i0 += 32) {
+                const int i = i0 + lane;
+                int b = a, c = 0;
+                if (i < a1) {
+                    const int2 e = g.adj[i];
+                    b = lab[e.x];
+                    c = (int)(e.y > cap ? cap : e.y);
+                }
+                if (b == big) into += c;
+                const unsigned m = __ballot_sync(0xffffffffu, b != a && b != big);
+                if (b != a && b != big) {
+                    const int at = held + __popc(m & ((1u << lane) - 1u));
+                    bkey[wid][at] = (u64)a * nc + (u64)b;
+                    bval[wid][at] = c;
+                }
+                held += __popc(m);
+                if (held > kOutBuf - 34) flush();
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) into += __shfl_xor_sync(0xffffffffu, into, o);
+            if (into > cap) into = cap;
+            if (into > 0) {
+                if (lane < 2) {
+                    bkey[wid][held + lane] = lane ? (u64)big * nc + (u64)a : (u64)a * nc + (u64)big;
+                    bval[wid][held + lane] = (int)into;
+                }
+                held += 2;
+                if (held > kOutBuf - 34) flush();
+            }
+        }
+    }
+    if (held) flush();
+}
+
 // raw input arcs: validate and emit (u, v, c) for u != v, c > 0 (w == nullptr:
 // every arc has weight 1)
 __global__ void __launch_bounds__(kThreads)
@@ -447,12 +527,42 @@ int min_degree(const DevGraph &g, Work &w, cudaStream_t s) {
 __global__ void k_zero_count(Status *st) {
     st->count = 0;
     st->count2 = 0;
+    st->wedges = 0;
+    st->closed = 0;
 }
 
 // largest arc weight (st->count) and number of rows with exactly two arcs
 // (st->count2): when max weight < lambda-hat, 2 * max weight <= delta and no
-// row has two arcs, PR1, PR2 and the degree-2 rule cannot unite anything
+// row has two arcs, PR1, PR2 and the degree-2 rule cannot unite anything.
+// The first blocks also probe kWedges wedges (two arcs of an evenly spaced
+// vertex): st->closed of the st->wedges found have their ends adjacent.  Above
+// one half the graph is clustered (hyperbolic graphs 0.75-0.77; R-MAT cores
+// 0.11-0.26, random graphs below 0.14, at every size looked at), and its
+// rounds are the scans'; else the forest packing's (mc_forest.cu).
+constexpr int kWedges = 1024;
+
 __global__ void k_graph_stats(const DevGraph g, Status *st) {
+    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < kWedges; k += gridDim.x * blockDim.x) {
+        const int u = (int)(((long long)k * g.n) / kWedges);
+        const int a0 = g.rp[u], len = g.rp[u + 1] - a0;
+        if (len < 2) continue;
+        const u64 h = splitmix64((u64)k);
+        const int i = (int)((h & 0xFFFFFFFFu) % (unsigned)len);
+        int j = (int)((h >> 32) % (unsigned)(len - 1));
+        j += j >= i;
+        const int v = g.adj[a0 + i].x, x = g.adj[a0 + j].x;
+        int lo = g.rp[v], hi = g.rp[v + 1] - 1;
+        bool closed = false;
+        while (lo <= hi && !closed) {
+            const int mid = (lo + hi) >> 1;
+            const int y = g.adj[mid].x;
+            closed = y == x;
+            if (y < x) lo = mid + 1;
+            else hi = mid - 1;
+        }
+        atomicAdd(&st->wedges, 1);
+        if (closed) atomicAdd(&st->closed, 1);
+    }
     int wmax = 0;
     long long two = 0;
     for (i64 j = (i64)blockIdx.x * blockDim.x + threadIdx.x; j < g.arcs; j += (i64)gridDim.x * blockDim.x)
@@ -523,7 +633,7 @@ static int build_from_pairs(i64 m, int nc, i64 clamp, int wb, DevGraph &out, Wor
 }
 
 int contract_graph(const DevGraph &in, DevGraph &out, Work &w, i64 clamp, bool flatten, int nc,
-                   cudaStream_t s, const std::function<int()> &post) {
+                   cudaStream_t s, const std::function<int()> &post, bool one_block) {
     const int n = in.n;
     // count2 (the emitted arcs) starts at 0: zeroed by the flatten, else here
     if (!flatten) { ++::mc::g_launches; k_zero_count<<<1, 1, 0, s>>>(w.st); }
@@ -541,9 +651,14 @@ int contract_graph(const DevGraph &in, DevGraph &out, Work &w, i64 clamp, bool f
     const int wb = bits_for((u64)(cap > 1 ? cap : 1));
     const int pack = (n >= 2 && bits_for((u64)n * (u64)n - 1) + wb <= 64) ? wb : 0;
     // block count (device) and emitted arcs in one status read
-    ++::mc::g_launches; k_emit<<<grid_for((in.arcs + kEmitItems - 1) / kEmitItems), kThreads, 0, s>>>(
-        in.src, in.adj, in.arcs, w.lab, (u64)nc, d_nc, clamp, pack, w.keysA, w.valsA,
-        reinterpret_cast<u64 *>(&w.st->count2), &w.st->err);
+    ++::mc::g_launches;
+    if (one_block && flatten && clamp <= (i64)kInt32Max)
+        k_emit_outside<<<grid_for(n), kThreads, 0, s>>>(in, w.lab, &w.st->giant, d_nc, clamp, pack, w.keysA, w.valsA,
+                                                        reinterpret_cast<u64 *>(&w.st->count2));
+    else
+        k_emit<<<grid_for((in.arcs + kEmitItems - 1) / kEmitItems), kThreads, 0, s>>>(
+            in.src, in.adj, in.arcs, w.lab, (u64)nc, d_nc, clamp, pack, w.keysA, w.valsA,
+            reinterpret_cast<u64 *>(&w.st->count2), &w.st->err);
     MC_CUDA(cudaGetLastError());
     MC_TRY(status_read(w, s));
     if (flatten) nc = (int)w.h_st->count;

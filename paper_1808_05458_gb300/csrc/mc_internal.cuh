@@ -94,7 +94,9 @@ struct Status {
     // graph creation: arcs running up and down, and a missing or unequal
     // mirror, seen while the input is built (valid when it is canonical)
     i64 sym_up, sym_down;
-    int sym_bad, pad_;
+    int sym_bad;
+    int giant;           // a vertex of the block most vertices are in (forest rounds)
+    int wedges, closed;  // wedges probed and closed (graph creation)
 };
 
 constexpr int kErrAsym = 1;       // asymmetric input
@@ -182,8 +184,9 @@ int status_read(Work &w, cudaStream_t s);
 // ready labels in [0, nc) with nc given.
 // `post` (may be empty) launches more work before the final status read,
 // whose Status copy the caller may then use; w.last_emitted = arcs emitted.
+// With `one_block` the block of st->giant holds most vertices of `in`.
 int contract_graph(const DevGraph &in, DevGraph &out, Work &w, i64 clamp, bool flatten, int nc,
-                   cudaStream_t s, const std::function<int()> &post = {});
+                   cudaStream_t s, const std::function<int()> &post = {}, bool one_block = false);
 
 // canonicalise raw CSR arrays (device) into `out` (drops self-loops / zero
 // weights, sums parallel arcs, sorts rows); checks symmetry if asked.
@@ -205,7 +208,8 @@ int connected_components(const DevGraph &g, Work &w, int *ncomp, cudaStream_t s)
 
 // minimum degree + smallest argmin into st->mindeg / st->argmin
 int min_degree(const DevGraph &g, Work &w, cudaStream_t s);
-// largest arc weight into st->count, rows with exactly two arcs into st->count2
+// largest arc weight into st->count, rows with exactly two arcs into
+// st->count2, probed wedges and how many are closed into st->wedges / closed
 int graph_stats(const DevGraph &g, Work &w, cudaStream_t s);
 
 // concurrent capped CAPFOREST (Alg. 1): unions into w.par, alpha updates
@@ -227,6 +231,13 @@ int capforest_full(const DevGraph &g, Work &w, const ScanConfig &cfg, cudaStream
 // true when capforest_full runs the one-warp scan of a small graph (n <= 8192,
 // bound <= 63, largest-key order), whose cost is a few wide scans'
 bool full_scan_is_small(int n, long long cap, bool fifo);
+
+// one round of certificates by forest packing at bound t (mc_forest.cu):
+// unions into w.par, their count into st->unions, a vertex of the largest
+// block into st->giant; the forests lie in w.keysA
+constexpr i64 kForestMaxT = 1024;
+bool forest_fits(const DevGraph &g, const Work &w, i64 t);
+int forest_round(const DevGraph &g, Work &w, i64 t, cudaStream_t s);
 
 // side bitmaps (original vertex ids, n0 bits)
 int side_from_vertex(Work &w, int n0, int vertex, cudaStream_t s);
