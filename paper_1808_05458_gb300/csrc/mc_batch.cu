@@ -130,6 +130,7 @@ struct BatchIn {
     Layout L;
     u64 seed;
     int pr_level;
+    int pr_late;  // the PR tests run only after a round that united little
     int fifo;
 };
 
@@ -995,14 +996,19 @@ __device__ long long pr_unions(P *par, const int *rpA, const int *srcA, const in
 // in-warp contraction, lambda-hat = min(., delta), until one vertex is left.
 // `lam` enters as lambda-hat and leaves as the minimum found; every lowering
 // rewrites the side bitmap S.best over the n0 vertices of S.orig.
+// With pr_late the PR tests wait for a round that united less than half of its
+// vertices: on most graphs the scans' own joins do that much, and the tests
+// cost more than they save, but on paths and cycles, where a scan may unite a
+// single edge, they are what ends the loop.
 template <int SN>
 __device__ void exact_rounds(Scratch &S, WarpSmem<SN> &sm, int n0, long long arcs, long long &lam, int &err,
-                             int &ovf, u64 seed, u64 tag, int pr_level, int fifo) {
+                             int &ovf, u64 seed, u64 tag, int pr_level, int pr_late, int fifo) {
     const int lane = lane_id();
     int n = n0;
     int *rpA = S.rpA, *srcA = S.srcA, *rpB = S.rpB, *srcB = S.srcB;
     int2 *adjA = S.adjA, *adjB = S.adjB;
     int round = 0, guard = 0;
+    bool poor = !pr_late;  // the last round united little (or the tests run every round)
     while (!err && n >= 2 && lam > 0) {
         if (++guard > 4 * n0 + 16) { err = MC_EINTERNAL; break; }
         const bool chip = round_on_chip<SN>(n, lam, fifo);
@@ -1014,7 +1020,7 @@ __device__ void exact_rounds(Scratch &S, WarpSmem<SN> &sm, int n0, long long arc
         __syncwarp();
         long long un = 0;
         // Padberg-Rinaldi PR1/PR2 and the degree-2 tie rule
-        if (pr_level >= 1) un = pr_unions(par32, rpA, srcA, adjA, S.deg, n, arcs, lam, pr_level);
+        if (pr_level >= 1 && poor) un = pr_unions(par32, rpA, srcA, adjA, S.deg, n, arcs, lam, pr_level);
         if (chip) {
             for (int v = lane; v < n; v += 32) par16[v] = (unsigned short)par32[v];
             __syncwarp();
@@ -1038,9 +1044,10 @@ __device__ void exact_rounds(Scratch &S, WarpSmem<SN> &sm, int n0, long long arc
                 return S.T[c] == 1 && S.order[c] < len;
             });
             lam = lam2;
-            if (un == 0) { ++round; continue; }
+            if (un == 0) { poor = true; ++round; continue; }
         }
         if (un == 0) { err = MC_EINTERNAL; break; }
+        poor = !pr_late || un * 2 < n;
         // contraction
         const int nc = chip ? warp_relabel(par16, S.root, S.lab, S.cnt, n) : warp_relabel(S.par, S.root, S.lab, S.cnt, n);
         // the result goes to the B buffers, then A and B swap roles
@@ -1286,7 +1293,7 @@ __device__ void solve_one(const BatchIn &B, int gi, Scratch &S, WarpSmem<SN> &sm
         warp_side_bits(S.best, n0, [&](int v) { return v == arg; });
         for (int v = lane; v < n0; v += 32) S.orig[v] = v;
         __syncwarp();
-        exact_rounds<SN>(S, sm, n0, arcs, lam, err, ovf, B.seed, (u64)gi, B.pr_level, B.fifo);
+        exact_rounds<SN>(S, sm, n0, arcs, lam, err, ovf, B.seed, (u64)gi, B.pr_level, B.pr_late, B.fifo);
     }
     if (lane == 0) {
         B.lam_out[gi] = lam;
@@ -1351,7 +1358,7 @@ __global__ void __launch_bounds__(32) k_tail(TailIn T) {
     __syncwarp();
     long long lam = T.lam;
     int err = 0, ovf = 0;
-    exact_rounds<SN>(S, sm, n, arcs, lam, err, ovf, T.seed, 0x7A11ULL, T.pr_level, T.fifo);
+    exact_rounds<SN>(S, sm, n, arcs, lam, err, ovf, T.seed, 0x7A11ULL, T.pr_level, 0, T.fifo);
     if (T.bits_out && lam < T.lam)
         for (int i = lane; i < (n + 31) / 32; i += 32) T.bits_out[i] = S.best[i];
     if (lane == 0) {
@@ -1414,6 +1421,18 @@ static const BatchShape kShapes[] = {{4, 1024, true},  {4, 2048, true},  {8, 512
                                      {8, 1024, false}, {2, 2048, false}};
 static int g_shape_choice = -1;  // -1: not tuned
 
+// The shape of a batch nobody tuned: the one whose warps hold the largest
+// graph on chip.  A graph that does not fit runs its scans from global memory:
+// 4096 graphs of 50 to 2000 vertices took 13.8 ms with room for 1024 on chip,
+// and take 4.1 ms with 2048.  Few graphs go two warps a block, so that each
+// has more of its SM (96 graphs of 50 to 400 vertices: 0.63 ms with eight warps
+// a block, 0.59 with two).  The PR tests of an untuned batch run late (see
+// exact_rounds).
+static int default_shape(int G, int nmax) {
+    if (nmax > 1022 || G <= 4 * num_sms()) return 4;  // {2, 2048}
+    return nmax > 510 ? 3 : 2;                        // {8, 1024}, {8, 512}
+}
+
 static int run_batch(int shape, BatchIn B, int warps, cudaStream_t s) {
     const BatchShape sh = kShapes[shape];
     if (sh.wpb == 4 && sh.sn == 1024) return launch_batch<4, 1024>(B, warps, s);
@@ -1467,7 +1486,9 @@ int batch_solve(int G, const long long *vtx_off, const long long *arc_off, const
         return arc_off[x + 1] - arc_off[x] > arc_off[y + 1] - arc_off[y];
     });
 
-    if (shape < 0) shape = g_shape_choice >= 0 ? g_shape_choice : 0;
+    if (shape < 0) shape = g_shape_choice;
+    const bool tuned = shape >= 0;
+    if (!tuned) shape = default_shape(G, nmax);
     const Layout L = make_layout(nmax, amax);
     const int wpb = kShapes[shape].wpb;
     const int warps_res = blocks_per_sm(shape) * wpb * num_sms();
@@ -1498,6 +1519,7 @@ int batch_solve(int G, const long long *vtx_off, const long long *arc_off, const
 
 
     BatchIn B;
+    memset(&B, 0, sizeof(B));  // compared bytewise below
     B.G = G;
     B.voff = (const long long *)(io + o_voff);
     B.aoff = (const long long *)(io + o_aoff);
@@ -1514,6 +1536,7 @@ int batch_solve(int G, const long long *vtx_off, const long long *arc_off, const
     B.L = L;
     B.seed = o.seed;
     B.pr_level = kShapes[shape].pr ? o.pr_level : 0;
+    B.pr_late = !tuned;
     B.fifo = o.pq_order == MC_PQ_FIFO;
 
     cudaEvent_t ea, eb;
