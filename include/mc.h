@@ -77,8 +77,9 @@ typedef struct mc_options {
     int32_t scans_per_round; /* concurrent CAPFOREST warps, 0 = auto.  Asking for
                                 something of the scans (this, region_budget,
                                 visits, MC_PQ_FIFO) has them run every round;
-                                else graphs that are not clustered take forest
-                                packing first                                  */
+                                else triangle tests (clustered graphs, with
+                                pr_level 4) or forest packing go first, and the
+                                scans run where these unite little             */
     int32_t region_budget;   /* max vertices touched by one scan, 0 = auto
                                 (192; 320 on graphs with >= 48 arcs/vertex;
                                 64 on graphs below 2^17 vertices)            */

@@ -1,10 +1,10 @@
 // mc_api.cu -- the C ABI (include/mc.h) and the host driver of Alg. 2.
 //
 // Driver per round on the current graph G_C (Alg. 2, Sec. 3.3):
-//   union-find reset -> Padberg-Rinaldi tests -> forest packing (mc_forest.cu)
-//   or, on clustered graphs and where it unites little, concurrent capped
-//   CAPFOREST (Alg. 1) -> if nothing was united: one full CAPFOREST scan
-//   (Alg. 3) ->
+//   union-find reset -> Padberg-Rinaldi tests -> triangle tests on clustered
+//   graphs (mc_pr.cu) or forest packing (mc_forest.cu) -> where they unite
+//   little, concurrent capped CAPFOREST (Alg. 1) -> if nothing was united: one
+//   full CAPFOREST scan (Alg. 3) ->
 //   contraction (Sec. 3.2) -> lambda-hat = min(lambda-hat, delta(G_C)).
 // Every improvement of lambda-hat snapshots its side as a bitmap over the
 // original vertices (Sec. 3.3): a scan's prefix for an alpha cut, the
@@ -463,10 +463,9 @@ int solve_impl(mc_graph *g, const mc_options &o, cudaStream_t s, SolveOut &out) 
     int rounds = 0, fallbacks = 0;
     const int tail_n = o.tail_vertices == 0 ? 256 : (o.tail_vertices > 4096 ? 4096 : o.tail_vertices);
     const bool verbose = getenv("MC_VERBOSE") != nullptr;
-// forest packing in place of the concurrent scans, unless the options ask
-    // for something of the scans (mc_forest.cu on which graphs gain by it)
-    const bool pack_forests = !g->clustered && o.pq_order != MC_PQ_FIFO && o.visits <= 1 && o.region_budget <= 0 &&
-                              o.scans_per_round <= 0;
+    // certificates without scans (mc_pr.cu, mc_forest.cu), unless the options
+    // ask for something of the scans
+    const bool quick = o.pq_order != MC_PQ_FIFO && o.visits <= 1 && o.region_budget <= 0 && o.scans_per_round <= 0;
 
     // Alg. 2's loop from `cur`, contracting into the free buffer of Ga / Gb;
     // lowers lam and records sides through w.orig
@@ -552,21 +551,41 @@ int solve_impl(mc_graph *g, const mc_options &o, cudaStream_t s, SolveOut &out) 
             return MC_OK;
         };
         i64 unions = 0;
-        // forest packing; a round of it that unites less than an eighth of the
-        // vertices has the scans try as well
-        bool packed = false;
-        if (pack_forests && forest_fits(cur, w, thr)) {
+        // the certificates that need no scan: triangles on a clustered input
+        // graph, else forest packing, also on what small graphs a clustered one
+        // was contracted to (a larger one still falls apart under it: of the
+        // 762 K vertices an RHG graph's first contraction left, the forests
+        // united four in five, the scans thirteen in fourteen).  A round that
+        // unites less than an eighth of the vertices has the scans try as well.
+        bool packed = false, one_block = false;
+        const bool input = cur.rp == g->G0.rp;
+        if (quick && g->clustered && input && o.pr_level >= 4 && thr < kTriMaxBound) {
+            MC_TRY(pr_triangles(cur, w, thr, g->wmax0 == 1, s));
+            MC_TRY(flatten_labels(w, cur.n, s));
+            MC_TRY(find_giant(w, cur.n, s));
+            MC_TRY(status_read(w, s));
+            unions = w.h_st->unions;
+            packed = unions * 8 >= cur.n;
+            one_block = w.h_st->giant_share >= 192;
+            // offsets, labels and the first arcs of every row, and about `thr`
+            // common neighbours in each of three tests' two rows
+            bytes += (i64)cur.n * (3 * 16 * thr + 3 * 64);
+            ph.mark(&S.ms_pr);
+        } else if (quick && (!g->clustered || (!input && cur.n < (1 << 17))) && forest_fits(cur, w, thr)) {
             MC_TRY(forest_round(cur, w, thr, s));
             MC_TRY(status_read(w, s));
             unions = w.h_st->unions;
             packed = unions * 8 >= cur.n;
+            one_block = unions * 2 >= cur.n;
             // heads of the rows, and each parent written once and read twice
             bytes += (i64)cur.n * thr * 20 + (i64)cur.n * 16;
-            if (verbose)
-                fprintf(stderr, "[mc] round %d n=%d arcs=%lld lam=%lld forests: unions=%lld\n", rounds, cur.n,
-                        (long long)cur.arcs, (long long)thr, (long long)unions);
         }
-        const bool one_block = packed && unions * 2 >= cur.n;
+        if (verbose && quick)
+            fprintf(stderr, "[mc] round %d n=%d arcs=%lld lam=%lld: unions=%lld without scans\n", rounds, cur.n,
+                    (long long)cur.arcs, (long long)thr, (long long)unions);
+        // reading the rows outside the largest block pays where there is much
+        // to leave out
+        one_block = one_block && packed && cur.arcs >= (1 << 20);
         if (!packed) MC_TRY(scan_round(cfg.budget, &unions));
         ph.mark(&S.ms_capforest);
         // a poor round: the triangle tests PR3/PR4 add their unions, on the

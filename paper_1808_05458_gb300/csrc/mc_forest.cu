@@ -61,43 +61,7 @@ struct Pack {
 
 __device__ __forceinline__ bool owns(int u, i64 du, int v, i64 dv) { return du < dv || (du == dv && u > v); }
 
-// the parent of x as this SM last saw it: an older parent is an ancestor all
-// the same (parents only move towards the root), so it may come from L1
-__device__ __forceinline__ int ld_parent(const int *p) {
-    int v;
-    asm volatile("ld.global.ca.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-
-__device__ __forceinline__ int root_of(const int *p, int x) {
-    while (true) {
-        const int q = ld_parent(p + x);
-        if (q == x) return x;
-        x = q;
-    }
-}
-
 __device__ __forceinline__ bool apart(const int *p, int a, int b) { return root_of(p, a) != root_of(p, b); }
-
-// links the larger root to the smaller one; false if the ends were connected.
-// What was read may be old: a root that is none any more fails its CAS (which
-// returns its parent as it is), and a node that was a root has a smaller root
-// now, so no cycle closes.
-__device__ __forceinline__ bool join(int *p, int a, int b) {
-    a = root_of(p, a);
-    b = root_of(p, b);
-    while (a != b) {
-        if (a < b) {
-            const int t = a;
-            a = b;
-            b = t;
-        }
-        const int old = atomicCAS(p + a, a, b);
-        if (old == a) return true;
-        a = root_of(p, old);
-    }
-    return false;
-}
 
 __device__ __forceinline__ unsigned mix32(unsigned x) {
     x ^= x >> 16;
@@ -242,7 +206,7 @@ __global__ void __launch_bounds__(kThreads) k_pack_join(const DevGraph g, Pack P
         if (!apart(p, u, v)) continue;
         const u32 bit = 1u << (i & 31);
         if (atomicOr(&P.taken[i >> 5], bit) & bit) continue;  // another forest has it
-        if (!join(p, u, v)) atomicAnd(&P.taken[i >> 5], ~bit);
+        if (!uf_join(p, u, v)) atomicAnd(&P.taken[i >> 5], ~bit);
     }
 }
 
@@ -408,7 +372,7 @@ k_pack_fill(const DevGraph g, Pack P, int *par, const int *__restrict__ reps, in
                     }
                 }
                 const int inc = warp_incl_sum(c), s = got + inc - c;
-                for (int x = s; x < s + c && x < nm; ++x) join(P.F + miss[x] * P.n, u, v);
+                for (int x = s; x < s + c && x < nm; ++x) uf_join(P.F + miss[x] * P.n, u, v);
                 got += __shfl_sync(0xffffffffu, inc, 31);
             }
             __syncwarp();

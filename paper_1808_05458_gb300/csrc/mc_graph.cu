@@ -245,84 +245,189 @@ k_emit(const int *__restrict__ src, const int2 *__restrict__ adj, i64 arcs, cons
     }
 }
 
-// The same arcs read from the rows outside one block that holds most of the
-// vertices: an arc from that block is the mirror of one of theirs.  A row's
-// weight into the block is added up (saturated like the rest) and emitted once
-// in both directions.  A warp a row; what a warp finds waits in shared memory
-// and goes out 64 or more at a time, one atomic each.  Against reading every
-// arc (10-core of an R-MAT graph, 29 M arcs, one block of all but a few
-// vertices): 105 -> 8 us.
-constexpr int kOutBuf = 128;
-
-__global__ void __launch_bounds__(kThreads)
-k_emit_outside(const DevGraph g, const int *__restrict__ lab, const int *giant, const int *d_nc, i64 clamp, int wb,
-               u64 *__restrict__ keys, int *__restrict__ vals, u64 *counter) {
-    __shared__ u64 bkey[kThreads / 32][kOutBuf];
-    __shared__ int bval[kThreads / 32][kOutBuf];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const u64 nc = (u64)*d_nc;
-    const int big = lab[*giant];
-    const long long cap = clamp < (i64)kInt32Max ? clamp : (i64)kInt32Max;
-    int held = 0;
-    auto flush = [&]() {
+// what a warp emits, held in shared memory until kOutBuf entries are near
+constexpr int kOutBuf = 256;
+struct OutBuf {
+    u64 key[kThreads / 32][kOutBuf];
+    int val[kThreads / 32][kOutBuf];
+};
+struct Emitter {
+    OutBuf *buf;
+    int wb, held;
+    u64 *keys;
+    int *vals;
+    u64 *counter;
+    // room for `want` more; all lanes call
+    __device__ __forceinline__ void room(int want) {
+        if (held + want <= kOutBuf) return;
+        const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
         __syncwarp();
         u64 base = 0;
         if (lane == 0) base = atomicAdd(counter, (u64)held);
         base = __shfl_sync(0xffffffffu, base, 0);
         for (int i = lane; i < held; i += 32) {
             if (wb) {
-                keys[base + i] = (bkey[wid][i] << wb) | (u64)(unsigned)bval[wid][i];
+                keys[base + i] = (buf->key[wid][i] << wb) | (u64)(unsigned)buf->val[wid][i];
             } else {
-                keys[base + i] = bkey[wid][i];
-                vals[base + i] = bval[wid][i];
+                keys[base + i] = buf->key[wid][i];
+                vals[base + i] = buf->val[wid][i];
             }
         }
         held = 0;
         __syncwarp();
-    };
-    const int nw = (gridDim.x * blockDim.x) >> 5;
-    for (int v0 = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32; v0 < g.n; v0 += nw * 32) {
-        const int vl = v0 + lane;
-        const int al = vl < g.n ? lab[vl] : big;
-        unsigned todo = __ballot_sync(0xffffffffu, al != big);
-        while (todo) {
-            const int l = __ffs(todo) - 1;
-            todo &= todo - 1;
-            const int u = v0 + l, a = __shfl_sync(0xffffffffu, al, l);
-            const int a1 = g.rp[u + 1];
-            long long into = 0;
-            for (int i0 = g.rp[u]; i0 < a1; i0 += 32) {
-                const int i = i0 + lane;
-                int b = a, c = 0;
-                if (i < a1) {
-                    const int2 e = g.adj[i];
-                    b = lab[e.x];
-                    c = (int)(e.y > cap ? cap : e.y);
-                }
-                if (b == big) into += c;
-                const unsigned m = __ballot_sync(0xffffffffu, b != a && b != big);
-                if (b != a && b != big) {
-                    const int at = held + __popc(m & ((1u << lane) - 1u));
-                    bkey[wid][at] = (u64)a * nc + (u64)b;
-                    bval[wid][at] = c;
-                }
-                held += __popc(m);
-                if (held > kOutBuf - 34) flush();
-            }
+    }
+    __device__ __forceinline__ void put(bool want, u64 key, int c) {
+        const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+        const unsigned m = __ballot_sync(0xffffffffu, want);
+        if (want) {
+            const int at = held + __popc(m & ((1u << lane) - 1u));
+            buf->key[wid][at] = key;
+            buf->val[wid][at] = c;
+        }
+        held += __popc(m);
+    }
+};
+
+// The same from a graph known to be symmetric: of an arc and its mirror only
+// the one to the smaller vertex is looked up, and what it gives goes out in
+// both directions (so that the output still fits the arcs' buffer).  Equal
+// keys of a warp's 32 arcs are added up wherever they stand, and a warp keeps
+// what it finds until it has some 200: with few arcs between blocks a pass is
+// the arcs read once and the labels' random sectors.  n = 2^20, 34 M arcs, 0.3 %
+// of them between blocks: 147 -> 88 us (k_emit's block-wide ranking with
+// only the lookups halved: 214).
+__global__ void __launch_bounds__(kThreads)
+k_emit_half(const int *__restrict__ src, const int2 *__restrict__ adj, i64 arcs, const int *__restrict__ lab,
+            u64 nc, const int *d_nc, i64 clamp, int wb, u64 *__restrict__ keys, int *__restrict__ vals, u64 *counter) {
+    constexpr unsigned kAll = 0xffffffffu;
+    constexpr int kU = 4;
+    __shared__ OutBuf buf;
+    if (d_nc) nc = (u64)*d_nc;
+    const int cap = (int)(clamp < (i64)kInt32Max ? clamp : (i64)kInt32Max);
+    const bool merge = cap < (1 << 26);  // 32 weights add up below 2^31
+    const int lane = threadIdx.x & 31;
+    const i64 step = (i64)gridDim.x * blockDim.x * kU;
+    Emitter out{&buf, wb, 0, keys, vals, counter};
+    for (i64 i0 = ((i64)blockIdx.x * blockDim.x + (threadIdx.x & ~31)) * kU; i0 < arcs; i0 += step) {
+        int u[kU], a[kU], b[kU];
+        int2 e[kU];
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) into += __shfl_xor_sync(0xffffffffu, into, o);
-            if (into > cap) into = cap;
-            if (into > 0) {
-                if (lane < 2) {
-                    bkey[wid][held + lane] = lane ? (u64)big * nc + (u64)a : (u64)a * nc + (u64)big;
-                    bval[wid][held + lane] = (int)into;
+        for (int k = 0; k < kU; ++k) {
+            const i64 i = i0 + 32 * k + lane;
+            u[k] = i < arcs ? src[i] : 0;
+            e[k] = i < arcs ? adj[i] : make_int2(INT_MAX, 0);
+        }
+#pragma unroll
+        for (int k = 0; k < kU; ++k) {
+            const bool down = e[k].x < u[k];
+            a[k] = down ? lab[u[k]] : 0;
+            b[k] = down ? lab[e[k].x] : 0;
+        }
+#pragma unroll
+        for (int k = 0; k < kU; ++k) {
+            const bool cross = a[k] != b[k];
+            if (!__any_sync(kAll, cross)) continue;
+            const u64 key = (u64)a[k] * nc + (u64)b[k];
+            int c = e[k].y < cap ? e[k].y : cap;
+            bool first = cross;
+            if (merge) {
+                const unsigned peers = __match_any_sync(kAll, cross ? key : ~(u64)lane);
+                if (cross) {
+                    const unsigned sum = __reduce_add_sync(peers, (unsigned)c);
+                    c = sum < (unsigned)cap ? (int)sum : cap;
+                    first = lane == __ffs(peers) - 1;
                 }
-                held += 2;
-                if (held > kOutBuf - 34) flush();
             }
+            out.room(64);
+            out.put(first, key, c);
+            out.put(first, (u64)b[k] * nc + (u64)a[k], c);
         }
     }
-    if (held) flush();
+    if (out.held) out.room(kOutBuf + 1);
+}
+
+// The same arcs read from the rows outside one block that holds most of the
+// vertices: an arc from that block is the mirror of one of theirs.  A row's
+// weight into the block is added up (saturated like the rest) and emitted once
+// in both directions.  Eight lanes a row (the whole warp a long one), `per`
+// (<= 32) rows looked over at a time.  Against reading every arc (10-core of an
+// R-MAT graph, 29 M arcs, one block of all but a few vertices): 105 -> 8 us.
+constexpr int kOutRow = 256;  // longer rows: the whole warp
+
+__global__ void __launch_bounds__(kThreads)
+k_emit_outside(const DevGraph g, const int *__restrict__ lab, const int *giant, const int *d_nc, i64 clamp, int wb,
+               int per, u64 *__restrict__ keys, int *__restrict__ vals, u64 *counter) {
+    constexpr unsigned kAll = 0xffffffffu;
+    constexpr int kU = 4;  // arcs a lane loads at once
+    __shared__ OutBuf buf;
+    const int lane = threadIdx.x & 31, gl = lane & 7, grp = lane >> 3;
+    const u64 nc = (u64)*d_nc;
+    const int big = lab[*giant];
+    const int cap = (int)(clamp < (i64)kInt32Max ? clamp : (i64)kInt32Max);
+    Emitter out{&buf, wb, 0, keys, vals, counter};
+    // lanes first, first + step, ... of a row: its weight into the block
+    auto walk = [&](int a, int i, int i1, int step) {
+        long long into = 0;
+        while (__any_sync(kAll, i < i1)) {
+            int2 e[kU];
+            int b[kU];
+#pragma unroll
+            for (int k = 0; k < kU; ++k) e[k] = i + k * step < i1 ? g.adj[i + k * step] : make_int2(-1, 0);
+#pragma unroll
+            for (int k = 0; k < kU; ++k) b[k] = e[k].x >= 0 ? lab[e[k].x] : a;
+#pragma unroll
+            for (int k = 0; k < kU; ++k) {
+                const int c = e[k].y < cap ? e[k].y : cap;
+                const bool other = b[k] != a && b[k] != big;
+                if (b[k] != a && b[k] == big) into += c;
+                if (__any_sync(kAll, other)) {
+                    out.room(32);
+                    out.put(other, (u64)a * nc + (u64)b[k], c);
+                }
+            }
+            i += kU * step;
+        }
+        return into;
+    };
+    auto put_into = [&](bool first, int a, long long into) {
+        const bool want = first && into > 0;
+        if (!__any_sync(kAll, want)) return;
+        const int c = (int)(into < cap ? into : cap);
+        out.room(64);
+        out.put(want, (u64)a * nc + (u64)big, c);
+        out.put(want, (u64)big * nc + (u64)a, c);
+    };
+    const int nw = (gridDim.x * blockDim.x) >> 5;
+    for (int v0 = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * per; v0 < g.n; v0 += nw * per) {
+        const int vl = v0 + lane;
+        const int al = lane < per && vl < g.n ? lab[vl] : big;
+        unsigned todo = __ballot_sync(kAll, al != big);
+        if (!todo) continue;
+        const int r0 = al != big ? g.rp[vl] : 0, r1 = al != big ? g.rp[vl + 1] : 0;
+        unsigned wide = __ballot_sync(kAll, r1 - r0 > kOutRow);
+        todo &= ~wide;
+        while (todo) {  // four rows at a time, eight lanes each
+            unsigned t = todo;
+            for (int k = 0; k < grp; ++k) t &= t - 1u;
+            for (int k = 0; k < 4; ++k) todo &= todo - 1u;
+            const int l = t ? __ffs(t) - 1 : 0;
+            const int a = __shfl_sync(kAll, al, l), s0 = __shfl_sync(kAll, r0, l), s1 = __shfl_sync(kAll, r1, l);
+            long long into = walk(a, t ? s0 + gl : 0, t ? s1 : 0, 8);
+#pragma unroll
+            for (int o = 4; o > 0; o >>= 1) into += __shfl_xor_sync(kAll, into, o);
+            put_into(t != 0u && gl == 0, a, into);
+        }
+        while (wide) {
+            const int l = __ffs(wide) - 1;
+            wide &= wide - 1u;
+            const int a = __shfl_sync(kAll, al, l), s0 = __shfl_sync(kAll, r0, l), s1 = __shfl_sync(kAll, r1, l);
+            long long into = walk(a, s0 + lane, s1, 32);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) into += __shfl_xor_sync(kAll, into, o);
+            put_into(lane == 0, a, into);
+        }
+    }
+    if (out.held) out.room(kOutBuf + 1);
 }
 
 // raw input arcs: validate and emit (u, v, c) for u != v, c > 0 (w == nullptr:
@@ -652,18 +757,27 @@ int contract_graph(const DevGraph &in, DevGraph &out, Work &w, i64 clamp, bool f
     const int pack = (n >= 2 && bits_for((u64)n * (u64)n - 1) + wb <= 64) ? wb : 0;
     // block count (device) and emitted arcs in one status read
     ++::mc::g_launches;
-    if (one_block && flatten && clamp <= (i64)kInt32Max)
-        k_emit_outside<<<grid_for(n), kThreads, 0, s>>>(in, w.lab, &w.st->giant, d_nc, clamp, pack, w.keysA, w.valsA,
-                                                        reinterpret_cast<u64 *>(&w.st->count2));
-    else
-        k_emit<<<grid_for((in.arcs + kEmitItems - 1) / kEmitItems), kThreads, 0, s>>>(
-            in.src, in.adj, in.arcs, w.lab, (u64)nc, d_nc, clamp, pack, w.keysA, w.valsA,
-            reinterpret_cast<u64 *>(&w.st->count2), &w.st->err);
+    u64 *emitted = reinterpret_cast<u64 *>(&w.st->count2);
+    const int eg = grid_for((in.arcs + kEmitItems - 1) / kEmitItems);
+    if (in.sym && one_block && flatten && clamp <= (i64)kInt32Max) {
+        // few enough vertices a warp that every warp has some
+        int per = n / (num_sms() * 64);
+        per = per < 1 ? 1 : (per > 32 ? 32 : per);
+        k_emit_outside<<<grid_for((i64)n * 32 / per), kThreads, 0, s>>>(in, w.lab, &w.st->giant, d_nc, clamp, pack, per,
+                                                                        w.keysA, w.valsA, emitted);
+    } else if (in.sym) {
+        k_emit_half<<<eg, kThreads, 0, s>>>(in.src, in.adj, in.arcs, w.lab, (u64)nc, d_nc, clamp, pack, w.keysA,
+                                            w.valsA, emitted);
+    } else {
+        k_emit<<<eg, kThreads, 0, s>>>(in.src, in.adj, in.arcs, w.lab, (u64)nc, d_nc, clamp, pack, w.keysA, w.valsA,
+                                       emitted, &w.st->err);
+    }
     MC_CUDA(cudaGetLastError());
     MC_TRY(status_read(w, s));
     if (flatten) nc = (int)w.h_st->count;
     const i64 m = w.h_st->count2;
     w.last_emitted = m;
+    out.sym = in.sym;
     return build_from_pairs(m, nc, clamp, pack, out, w, s, post);
 }
 
@@ -818,6 +932,7 @@ int canonicalize(int n, const int *rp, const int *col, const int *w, bool check_
     if (wk.h_st->err) return MC_EINVAL;
     out.n = n;
     out.arcs = arcs_raw;
+    out.sym = check_sym;  // or the check below fails
     const bool canonical_input = wk.h_st->count2 == 0;
     if (!canonical_input) {
         ++::mc::g_launches; k_zero_count<<<1, 1, 0, s>>>(wk.st);
@@ -988,6 +1103,38 @@ namespace mc {
 
 int flatten_labels(Work &w, int n, cudaStream_t s) {
     ++::mc::g_launches; k_flatten<<<grid_for(n), kThreads, 0, s>>>(w.par, w.root, w.cnt, n, nullptr);
+    MC_CUDA(cudaGetLastError());
+    return MC_OK;
+}
+
+__global__ void __launch_bounds__(256) k_giant(const int *__restrict__ root, int n, Status *st) {
+    constexpr int kH = 512;
+    __shared__ int key[kH], cnt[kH];
+    __shared__ unsigned long long best;
+    for (int i = threadIdx.x; i < kH; i += blockDim.x) {
+        key[i] = -1;
+        cnt[i] = 0;
+    }
+    if (threadIdx.x == 0) best = 0;
+    __syncthreads();
+    const int r = root[(int)(((long long)threadIdx.x * n) >> 8)];
+    unsigned h = ((unsigned)r * 2654435761u) >> 23;
+    while (true) {
+        const int k = atomicCAS(&key[h], -1, r);
+        if (k == -1 || k == r) break;
+        h = (h + 1) & (kH - 1);
+    }
+    const int c = atomicAdd(&cnt[h], 1) + 1;
+    atomicMax(&best, ((unsigned long long)c << 32) | (unsigned)(INT_MAX - r));
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        st->giant = INT_MAX - (int)(best & 0xFFFFFFFFu);
+        st->giant_share = (int)(best >> 32);
+    }
+}
+
+int find_giant(Work &w, int n, cudaStream_t s) {
+    ++::mc::g_launches; k_giant<<<1, 256, 0, s>>>(w.root, n, w.st);
     MC_CUDA(cudaGetLastError());
     return MC_OK;
 }

@@ -71,6 +71,7 @@ struct DevGraph {
     int *src = nullptr;
     int2 *adj = nullptr;
     i64 *deg = nullptr;
+    bool sym = false;  // every arc is known to have its mirror (not for trusted input)
 };
 
 // Device-resident status block, read back once per phase.
@@ -96,6 +97,7 @@ struct Status {
     i64 sym_up, sym_down;
     int sym_bad;
     int giant;           // a vertex of the block most vertices are in (forest rounds)
+    int giant_share;     // how many of the 256 vertices find_giant looks at are in it
     int wedges, closed;  // wedges probed and closed (graph creation)
 };
 
@@ -249,6 +251,13 @@ int orig_update(Work &w, int n0, cudaStream_t s);           // orig = lab[orig]
 // (every edge if budget < 0)
 int pr_tests_budget(const DevGraph &g, Work &w, i64 lam, int lo, int level, int budget,
                     cudaStream_t s);
+// PR1/PR4 on a few arcs of every row (clustered graphs; bounds below
+// kTriMaxBound); unit: every weight of g is 1
+constexpr i64 kTriMaxBound = 1 << 26;
+int pr_triangles(const DevGraph &g, Work &w, i64 lam, bool unit, cudaStream_t s);
+// a vertex of the block that most of 256 evenly spaced vertices are in ->
+// st->giant, their share (of 256) -> st->giant_share; w.root from a flatten
+int find_giant(Work &w, int n, cudaStream_t s);
 int flatten_labels(Work &w, int n, cudaStream_t s);   // w.root[v] = root of v in w.par
 int round_reset(Work &w, i64 lam, cudaStream_t s);    // st->lam = lam, counters = 0
 int round_start(Work &w, int n, i64 lam, cudaStream_t s);  // union_find_init + round_reset
@@ -334,6 +343,45 @@ __device__ __forceinline__ int uf_find(int *par, int x) {
         p[x] = gx;
         x = gx;
     }
+}
+
+// the parent of x as this SM last saw it: an older parent is an ancestor all
+// the same (parents only move towards the root), so it may come from L1.  It
+// should where many threads walk to one root: a million warps that fetch that
+// root's word from L2 wait for its one slice (k_tri_* in
+// mc_pr.cu)
+__device__ __forceinline__ int ld_parent(const int *p) {
+    int v;
+    asm volatile("ld.global.ca.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+
+__device__ __forceinline__ int root_of(const int *p, int x) {
+    while (true) {
+        const int q = ld_parent(p + x);
+        if (q == x) return x;
+        x = q;
+    }
+}
+
+// links the larger root to the smaller one; false if the ends were connected.
+// What was read may be old: a root that is none any more fails its CAS (which
+// returns its parent as it is), and a node that was a root has a smaller root
+// now, so no cycle closes.
+__device__ __forceinline__ bool uf_join(int *p, int a, int b) {
+    a = root_of(p, a);
+    b = root_of(p, b);
+    while (a != b) {
+        if (a < b) {
+            const int t = a;
+            a = b;
+            b = t;
+        }
+        const int old = atomicCAS(p + a, a, b);
+        if (old == a) return true;
+        a = root_of(p, old);
+    }
+    return false;
 }
 
 // as uf_union; *root = the root of the merged set (its smallest member)

@@ -230,6 +230,222 @@ k_pr34_pairs(const DevGraph g, int *par, long long lam, int lo, int level, int m
     if (local) atomicAdd(unions, (unsigned long long)local);
 }
 
+// PR4 (and PR1) on a few arcs of every row.  In a clustered graph almost any
+// edge has the common neighbours to pass, and two united edges a vertex leave
+// hardly a block of its own, so a few tests a vertex do what otherwise takes a
+// scan of every arc: every vertex tests its first arc, then its second if that
+// runs between two blocks by then, then one of its first eight that does.
+//
+// Eight lanes a test: they hold eight arcs of either row, compare them all by
+// shuffles, and go on with the next eight of the row whose ids end first, until
+// the common weight reaches the bound (or for a number of steps: what is
+// counted then is a lower bound, so the test only gets weaker).  Bound by
+// latency (offsets, arcs, parents, one after another; issue slots 44 % used)
+// and by the neighbours' sectors.  The round against one of concurrent scans,
+// hyperbolic graphs: n = 2^20, 34 M arcs, bound 6: 0.88 -> 0.32 ms; n = 2^22,
+// 268 M arcs, bound 20: 5.5 -> 2.0 ms.  What was slower: a thread a test (it
+// walks the rows one arc at a time, and the lines of a thousand walks a SM push
+// each other out of L1: 1.2 ms at n = 2^20); sixteen arcs a step (twice the
+// sectors for a bound of 6: the first pass 132 -> 152 us); parents read past L1
+// (the common root's word comes from one L2 slice: the last pass 0.63 ms of
+// 0.04); tests in place of the job lists (warps with several tests at the end:
+// 0.12 ms of 0.02); one atomic a warp on the union counter over a full grid
+// (0.28 ms of 0.11).
+//
+// UNIT: every weight is 1, so a common neighbour counts 1.
+struct TriJob {
+    int u, v, c;
+};
+
+// one test a group of eight lanes (u < 0: none); the common weight, `need` at most
+template <bool UNIT>
+__device__ __forceinline__ int tri_test(const DevGraph &g, TriJob t, int need, int max_steps) {
+    constexpr unsigned kAll = 0xffffffffu;
+    const int gl = threadIdx.x & 7;
+    const int2 none = make_int2(INT_MAX, 0);
+    int i = 0, i1 = 0, j = 0, j1 = 0;
+    if (t.u >= 0) {
+        i = g.rp[t.u];
+        i1 = g.rp[t.u + 1];
+        j = g.rp[t.v];
+        j1 = g.rp[t.v + 1];
+    }
+    int2 x = i + gl < i1 ? g.adj[i + gl] : none, y = j + gl < j1 ? g.adj[j + gl] : none;
+    int sum = t.c < need ? t.c : need;
+    bool act = t.u >= 0 && sum < need;
+    for (int st = 0; st < max_steps && __any_sync(kAll, act); ++st) {
+        int m;
+        if (UNIT) {
+            bool h = false;
+#pragma unroll
+            for (int s = 0; s < 8; ++s) h |= __shfl_sync(kAll, y.x, s, 8) == x.x;
+            m = __popc(__ballot_sync(kAll, h && x.x != INT_MAX) & (0xffu << (threadIdx.x & 24)));
+        } else {
+            int hit = -1;
+#pragma unroll
+            for (int s = 0; s < 8; ++s)
+                if (__shfl_sync(kAll, y.x, s, 8) == x.x) hit = s;
+            const int wy = __shfl_sync(kAll, y.y, hit & 7, 8);
+            m = hit >= 0 && x.x != INT_MAX ? (x.y < wy ? x.y : wy) : 0;
+            m = m < need ? m : need;
+#pragma unroll
+            for (int o = 1; o < 8; o <<= 1) m += __shfl_xor_sync(kAll, m, o, 8);
+        }
+        // the row whose ids end first goes on; when it has no more, no common
+        // neighbour is left
+        const int ex = __shfl_sync(kAll, x.x, i1 - i < 8 ? (i1 - i - 1) & 7 : 7, 8);
+        const int ey = __shfl_sync(kAll, y.x, j1 - j < 8 ? (j1 - j - 1) & 7 : 7, 8);
+        if (act) {
+            sum = m < need - sum ? sum + m : need;
+            if (ex <= ey) {
+                i += 8;
+                act = sum < need && i < i1;
+                if (act) x = i + gl < i1 ? g.adj[i + gl] : none;
+            } else {
+                j += 8;
+                act = sum < need && j < j1;
+                if (act) y = j + gl < j1 ? g.adj[j + gl] : none;
+            }
+        }
+    }
+    return sum;
+}
+
+__device__ __forceinline__ void tri_count(int local, unsigned long long *unions) {
+    local = (int)__reduce_add_sync(0xffffffffu, (unsigned)local);
+    if ((threadIdx.x & 31) == 0 && local) atomicAdd(unions, (unsigned long long)local);
+}
+
+// every vertex's first arc.  Its end is mostly smaller, and then the vertex
+// hangs from it without a find (parents stay smaller than their children).
+template <bool UNIT>
+__global__ void __launch_bounds__(256, 8)
+k_tri_first(const DevGraph g, int *par, int need, int max_steps, unsigned long long *unions) {
+    int local = 0;
+    for (i64 k = ((i64)blockIdx.x * blockDim.x + threadIdx.x) >> 3; (k & ~3) < g.n; k += (i64)gridDim.x * blockDim.x / 8) {
+        const int u = (int)k;
+        TriJob t{-1, 0, 0};
+        if (u < g.n) {
+            const int a = g.rp[u];
+            if (a < g.rp[u + 1]) {
+                const int2 e = g.adj[a];
+                t = TriJob{u, e.x, e.y};
+            }
+        }
+        const int sum = tri_test<UNIT>(g, t, need, max_steps);
+        if (t.u >= 0 && sum >= need && (threadIdx.x & 7) == 0) {
+            if (t.v < u && atomicCAS(&par[u], u, t.v) == u) ++local;
+            else local += uf_join(par, u, t.v);
+        }
+        __syncwarp();
+    }
+    tri_count(local, unions);
+}
+
+// every vertex points at its root
+__global__ void k_par_flatten(int *par, int n) {
+    for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
+        const int p = ld_parent(par + v), r = root_of(par, p);
+        if (r != p) par[v] = r;
+    }
+}
+
+// the jobs of the next pass: of each vertex the first of its first eight arcs
+// whose end is in another block (parents are roots here); (vertex << 32 | arc)
+__global__ void __launch_bounds__(256)
+k_tri_collect(const DevGraph g, const int *__restrict__ par, int q1, u64 *jobs, u64 *count) {
+    constexpr unsigned kAll = 0xffffffffu;
+    constexpr int kV = 4;  // vertices a group of eight lanes looks over at once
+    const int lane = threadIdx.x & 31, gl = lane & 7, grp = lane >> 3;
+    const int u0 = (int)(((i64)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 4 * kV;
+    int a0[kV], a1[kV], v[kV], pu[kV];
+#pragma unroll
+    for (int k = 0; k < kV; ++k) {
+        const int u = u0 + 4 * k + grp;
+        a0[k] = u < g.n ? g.rp[u] : 0;
+        a1[k] = u < g.n ? g.rp[u + 1] : 0;
+        pu[k] = u < g.n ? par[u] : -1;
+    }
+#pragma unroll
+    for (int k = 0; k < kV; ++k) v[k] = gl < q1 && a0[k] + gl < a1[k] ? g.adj[a0[k] + gl].x : -1;
+    int pos[kV], total = 0;
+#pragma unroll
+    for (int k = 0; k < kV; ++k) {
+        const bool open = v[k] >= 0 && par[v[k]] != pu[k];
+        const unsigned mine = (__ballot_sync(kAll, open) >> (lane & 24)) & 0xffu;
+        pos[k] = mine ? a0[k] + __ffs(mine) - 1 : -1;
+        total += mine != 0u && gl == 0;
+    }
+    int inc = total;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(kAll, inc, o);
+        if (lane >= o) inc += t;
+    }
+    // one global atomic a block
+    __shared__ int wsum[8];
+    __shared__ u64 s_base;
+    if (lane == 31) wsum[threadIdx.x >> 5] = inc;
+    __syncthreads();
+    int before = 0;
+    for (int w = 0; w < (int)(threadIdx.x >> 5); ++w) before += wsum[w];
+    if (threadIdx.x == 255) s_base = before + inc > 0 ? atomicAdd(count, (u64)(before + inc)) : 0;
+    __syncthreads();
+    u64 base = s_base + (u64)(before + inc - total);
+    if (gl == 0) {
+#pragma unroll
+        for (int k = 0; k < kV; ++k)
+            if (pos[k] >= 0) jobs[base++] = ((u64)(u32)(u0 + 4 * k + grp) << 32) | (u32)pos[k];
+    }
+}
+
+template <bool UNIT>
+__global__ void __launch_bounds__(256, 8)
+k_tri_jobs(const DevGraph g, int *par, const u64 *__restrict__ jobs, const u64 *count, int need, int max_steps,
+           unsigned long long *unions) {
+    const i64 nj = (i64)*count;
+    const i64 step = (i64)gridDim.x * blockDim.x / 8;
+    int local = 0;
+    for (i64 k0 = ((i64)blockIdx.x * blockDim.x + (threadIdx.x & ~31)) / 8; k0 < nj; k0 += step) {
+        const i64 k = k0 + ((threadIdx.x & 31) >> 3);
+        TriJob t{-1, 0, 0};
+        if (k < nj) {
+            const u64 job = jobs[k];
+            const int2 e = g.adj[(u32)job];
+            t = TriJob{(int)(job >> 32), e.x, e.y};
+        }
+        const int sum = tri_test<UNIT>(g, t, need, max_steps);
+        if (t.u >= 0 && sum >= need && (threadIdx.x & 7) == 0) local += uf_join(par, t.u, t.v);
+        __syncwarp();
+    }
+    tri_count(local, unions);
+}
+
+template <bool UNIT>
+static void launch_triangles(const DevGraph &g, Work &w, int need, cudaStream_t s) {
+    const int max_steps = 16 + (need < 4096 ? need : 4096);
+    auto *un = reinterpret_cast<unsigned long long *>(&w.st->unions);
+    u64 *count = reinterpret_cast<u64 *>(&w.st->count), *jobs = w.keysA;
+    int fb = (g.n + 255) / 256, jb = (int)(((i64)g.n * 8 + 255) / 256);
+    if (jb > num_sms() * 8) jb = num_sms() * 8;
+    ++::mc::g_launches; k_tri_first<UNIT><<<jb, 256, 0, s>>>(g, w.par, need, max_steps, un);
+    if (fb > num_sms() * 8) fb = num_sms() * 8;
+    for (int pass = 0; pass < 2; ++pass) {
+        ++::mc::g_launches; k_par_flatten<<<fb, 256, 0, s>>>(w.par, g.n);
+        cudaMemsetAsync(count, 0, sizeof(u64), s);
+        ++::mc::g_launches; k_tri_collect<<<(int)(((i64)g.n * 2 + 255) / 256), 256, 0, s>>>(g, w.par, pass ? 8 : 2, jobs, count);
+        ++::mc::g_launches; k_tri_jobs<UNIT><<<jb, 256, 0, s>>>(g, w.par, jobs, count, need, max_steps, un);
+    }
+}
+
+int pr_triangles(const DevGraph &g, Work &w, i64 lam, bool unit, cudaStream_t s) {
+    if (lam >= kTriMaxBound || g.arcs == 0) return MC_OK;
+    if (unit) launch_triangles<true>(g, w, (int)lam, s);
+    else launch_triangles<false>(g, w, (int)lam, s);
+    MC_CUDA(cudaGetLastError());
+    return MC_OK;
+}
+
 int pr_tests_budget(const DevGraph &g, Work &w, i64 lam, int lo, int level, int budget,
                     cudaStream_t s) {
     if (level <= 0 || lo > level || g.arcs == 0) return MC_OK;
