@@ -1608,7 +1608,8 @@ int tail_solve(const DevGraph &g, Work &w, int limit, long long *lam, u64 seed, 
                int n0, cudaStream_t s) {
     if (limit > 4096) limit = 4096;
     if (g.n > limit || g.arcs > 64LL * limit || g.n < 2) return MC_EINVAL;
-    const bool on_chip = g.n <= kTailSmemN && g.arcs <= kTailSmemArcs;
+    const bool dense = g.n <= kDenseN && *lam <= kDenseMaxLam && !fifo;
+    const bool on_chip = dense || (g.n <= kTailSmemN && g.arcs <= kTailSmemArcs);
     const Layout L = on_chip ? make_layout(kTailSmemN, kTailSmemArcs) : make_layout(limit, 64LL * limit);
     // the side bitmap is read back from global memory in both cases
     const size_t need = on_chip ? al(4 * ((size_t)kTailSmemN / 32 + 2)) : L.bytes;
@@ -1629,7 +1630,9 @@ int tail_solve(const DevGraph &g, Work &w, int limit, long long *lam, u64 seed, 
     T.fifo = fifo;
     T.out = w.st;
     T.bits_out = on_chip ? reinterpret_cast<u32 *>(w.tail) : nullptr;
-    if (on_chip) {
+    if (dense) {
+        MC_TRY(dense_solve(g, *lam, seed, pr_level, w.st, T.bits_out, s));
+    } else if (on_chip) {
         static bool attr = false;
         if (!attr) {
             MC_CUDA(cudaFuncSetAttribute(k_tail<kTailSmemSN, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,

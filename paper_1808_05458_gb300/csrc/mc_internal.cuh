@@ -294,6 +294,12 @@ int batch_shapes();
 // round); *lam = min(*lam, lambda(g)), the side recorded through w.orig
 int tail_solve(const DevGraph &g, Work &w, int limit, long long *lam, u64 seed, int pr_level, int fifo,
                int n0, cudaStream_t s);
+// the same on a dense matrix in shared memory (mc_dense.cu): at most kDenseN
+// vertices, a bound of at most kDenseMaxLam, the largest-key order; the bound
+// found into out->lam, a lower one's side into bits_out
+constexpr int kDenseN = 224;
+constexpr i64 kDenseMaxLam = (1 << 22) - 1;  // a column adds up below 2^30, a key's entry below 2^31
+int dense_solve(const DevGraph &g, i64 lam, u64 seed, int pr_level, Status *out, u32 *bits_out, cudaStream_t s);
 int side_from_bits(Work &w, int n0, const u32 *bits, cudaStream_t s);  // bit v = bits[orig[v]]
 void batch_set_shape(int shape);
 int batch_get_shape();
