@@ -54,36 +54,98 @@ __device__ __forceinline__ float u01s(u64 h) { return (float)((h >> 40) & 0xFFFF
 // double precision: once the walk has evened a side out, centring leaves a
 // small remainder of a large common value, which single precision would not
 // resolve.
-__global__ void k_rand_init(int n, u64 seed, double2 *__restrict__ S) {
-    for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
+// beside them what the passes over arcs need of every degree: 1 / d in double
+// (0 without arcs), d and 1 / d in float
+__global__ void k_rand_init(DevGraph g, u64 seed, double2 *__restrict__ S, double *__restrict__ rd,
+                            float2 *__restrict__ fd) {
+    for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < g.n; v += gridDim.x * blockDim.x) {
         const u64 h = splitmix64(seed ^ splitmix64((u64)(unsigned)v));
         S[v] = make_double2(2.0 * (double)u01s(h) - 1.0, 2.0 * (double)u01s(splitmix64(h)) - 1.0);
+        const i64 d = g.deg[v];
+        rd[v] = d > 0 ? 1.0 / (double)d : 0.0;
+        fd[v] = make_float2((float)d, d > 0 ? 1.f / (float)d : 0.f);
     }
 }
 
-// one lazy random-walk step: out = (in + D^-1 A in) / 2 (a vertex without
-// arcs keeps in / 2); one warp per vertex
-__global__ void k_smooth(DevGraph g, const double2 *__restrict__ in, double2 *__restrict__ out) {
-    const int lane = threadIdx.x & 31;
-    const int nw = (gridDim.x * blockDim.x) >> 5;
-    for (int v = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; v < g.n; v += nw) {
-        double sx = 0.0, sy = 0.0;
-        for (int i = g.rp[v] + lane; i < g.rp[v + 1]; i += 32) {
-            const int2 e = g.adj[i];
-            const double2 x = in[e.x];
-            sx += (double)e.y * x.x;
-            sy += (double)e.y * x.y;
+// One lazy random-walk step: out = (in + D^-1 A in) / 2 (a vertex without arcs
+// keeps in / 2).  Bound by the FP64 pipe, where a warp instruction takes 16
+// cycles of a SM whatever lanes it serves: eight lanes a vertex, so that a warp
+// reduces and finishes four vertices with the instructions of one (even lanes
+// the first sum, odd lanes the second), the reciprocals taken once before the
+// first step, and weights of 1 not converted.  A row of more than kLongRow
+// arcs gets the whole warp.  32768 vertices, 1 M arcs: 80 us a step with a warp
+// a vertex, 20 so (four lanes a vertex: 24).
+constexpr int kLongRow = 128;
+constexpr int kSmoothLg = 3;  // eight lanes a vertex
+
+__device__ __forceinline__ void smooth_arcs(const DevGraph &g, const double2 *__restrict__ in, int i, int i1, int step,
+                                            double &sx, double &sy) {
+        constexpr int kU = 4;
+    for (; __any_sync(0xffffffffu, i < i1); i += kU * step) {
+        int2 e[kU];
+        double2 x[kU];
+        bool unit = true;
+#pragma unroll
+        for (int k = 0; k < kU; ++k) {
+            e[k] = i + k * step < i1 ? g.adj[i + k * step] : make_int2(-1, 1);
+            unit &= e[k].y == 1;
         }
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            sx += __shfl_xor_sync(0xffffffffu, sx, o);
-            sy += __shfl_xor_sync(0xffffffffu, sy, o);
+        for (int k = 0; k < kU; ++k) x[k] = e[k].x >= 0 ? in[e[k].x] : make_double2(0.0, 0.0);
+        if (__all_sync(0xffffffffu, unit)) {
+#pragma unroll
+            for (int k = 0; k < kU; ++k) {
+                sx += x[k].x;
+                sy += x[k].y;
+            }
+        } else {
+#pragma unroll
+            for (int k = 0; k < kU; ++k) {
+                const double w = (double)e[k].y;
+                sx += w * x[k].x;
+                sy += w * x[k].y;
+            }
         }
-        if (lane == 0) {
-            const double d = (double)g.deg[v];
-            const double2 x = in[v];
-            out[v] = d > 0 ? make_double2(0.5 * (x.x + sx / d), 0.5 * (x.y + sy / d))
-                           : make_double2(0.5 * x.x, 0.5 * x.y);
+    }
+}
+
+// the two sums over 2^LG lanes: even lanes end with the first, odd lanes with
+// the second
+template <int LG>
+__device__ __forceinline__ double reduce_pair(double sx, double sy) {
+    const bool odd = threadIdx.x & 1;
+    const double give = odd ? sx : sy;
+    double s = (odd ? sy : sx) + __shfl_xor_sync(0xffffffffu, give, 1);
+#pragma unroll
+    for (int o = 2; o < (1 << LG); o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    return s;
+}
+
+__global__ void __launch_bounds__(256)
+k_smooth(DevGraph g, const double2 *__restrict__ in, const double *__restrict__ rd, double2 *__restrict__ out) {
+    constexpr int kLg = 1 << kSmoothLg, kPer = 32 / kLg;  // lanes a vertex, vertices a warp
+    const int lane = threadIdx.x & 31, sub = lane & (kLg - 1);
+    const double *in1 = reinterpret_cast<const double *>(in);
+    double *out1 = reinterpret_cast<double *>(out);
+    const int nw = (gridDim.x * blockDim.x) >> 5;
+    for (int v0 = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * kPer; v0 < g.n; v0 += nw * kPer) {
+        const int v = v0 + (lane >> kSmoothLg);
+        const int a0 = v < g.n ? g.rp[v] : 0, a1 = v < g.n ? g.rp[v + 1] : 0;
+        const bool longrow = a1 - a0 > kLongRow;
+        double sx = 0.0, sy = 0.0;
+        smooth_arcs(g, in, a0 + sub, longrow ? 0 : a1, kLg, sx, sy);
+        const double s = reduce_pair<kSmoothLg>(sx, sy);
+        if (v < g.n && sub < 2 && !longrow)
+            out1[2 * (size_t)v + sub] = 0.5 * (in1[2 * (size_t)v + sub] + s * rd[v]);
+        unsigned todo = __ballot_sync(0xffffffffu, longrow && sub == 0);
+        while (todo) {
+            const int l = __ffs(todo) - 1;
+            todo &= todo - 1u;
+            const int u = v0 + (l >> kSmoothLg);
+            double tx = 0.0, ty = 0.0;
+            smooth_arcs(g, in, __shfl_sync(0xffffffffu, a0, l) + lane, __shfl_sync(0xffffffffu, a1, l), 32, tx, ty);
+            const double t = reduce_pair<5>(tx, ty);
+            if (lane < 2) out1[2 * (size_t)u + lane] = 0.5 * (in1[2 * (size_t)u + lane] + t * rd[u]);
         }
     }
 }
@@ -118,12 +180,19 @@ __global__ void __launch_bounds__(256) k_center_partial(DevGraph g, const double
 // cs[0..1] = the degree-weighted means; the largest magnitudes of the
 // centred vectors go to cs[2..3] (as double bits, via integer maxima of
 // non-negative doubles) in k_maxabs
-__global__ void k_center_final(const double *__restrict__ part, int nb, double *cs) {
+// (one block; a fixed tree over the nb <= 256 partials)
+__global__ void __launch_bounds__(256) k_center_final(const double *__restrict__ part, int nb, double *cs) {
+    __shared__ double sh[3][256];
+    for (int j = 0; j < 3; ++j) sh[j][threadIdx.x] = (int)threadIdx.x < nb ? part[3 * threadIdx.x + j] : 0.0;
+    for (int o = 128; o > 0; o >>= 1) {
+        __syncthreads();
+        if ((int)threadIdx.x < o)
+            for (int j = 0; j < 3; ++j) sh[j][threadIdx.x] += sh[j][threadIdx.x + o];
+    }
     if (threadIdx.x == 0) {
-        double a = 0, b = 0, c = 0;
-        for (int k = 0; k < nb; ++k) { a += part[3 * k]; b += part[3 * k + 1]; c += part[3 * k + 2]; }
-        cs[0] = c > 0 ? a / c : 0.0;
-        cs[1] = c > 0 ? b / c : 0.0;
+        const double c = sh[2][0];
+        cs[0] = c > 0 ? sh[0][0] / c : 0.0;
+        cs[1] = c > 0 ? sh[1][0] / c : 0.0;
         cs[2] = 0.0;
         cs[3] = 0.0;
     }
@@ -146,9 +215,19 @@ __global__ void k_maxabs(int n, const double2 *__restrict__ S, double *cs) {
     }
 }
 
-__global__ void k_features(DevGraph g, long long delta, const double2 *__restrict__ Sm, const double *__restrict__ cs,
-                           const float *__restrict__ P, float *__restrict__ X, __nv_bfloat16 *__restrict__ H0,
-                           float *__restrict__ Z0) {
+// x_6 and x_7, a thread a vertex: a warp a vertex (k_features) would run the
+// double-precision divisions once for every vertex, not once for 32
+__global__ void k_scaled(int n, const double2 *__restrict__ Sm, const double *__restrict__ cs, float *__restrict__ X) {
+    for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
+        const double2 q = Sm[v];
+        const float x6 = (float)(cs[2] > 0.0 ? (q.x - cs[0]) / cs[2] : q.x - cs[0]);
+        const float x7 = (float)(cs[3] > 0.0 ? (q.y - cs[1]) / cs[3] : q.y - cs[1]);
+        *reinterpret_cast<float2 *>(X + (size_t)v * kF + 6) = make_float2(x6, x7);
+    }
+}
+
+__global__ void k_features(DevGraph g, long long delta, const float *__restrict__ P, float *__restrict__ X,
+                           __nv_bfloat16 *__restrict__ H0, float *__restrict__ Z0) {
     const int lane = threadIdx.x & 31;
     const int nw = (gridDim.x * blockDim.x) >> 5;
     for (int v = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; v < g.n; v += nw) {
@@ -176,10 +255,10 @@ __global__ void k_features(DevGraph g, long long delta, const double2 *__restric
         x[3] = (rel < 8.f ? rel : 8.f) / 8.f;
         x[4] = log1pf(a > 0 ? (float)sum / (float)a : 0.f) / 8.f;
         x[5] = log1pf(a > 0 ? (float)mn : 0.f) / 8.f;
-        const double2 q = Sm[v];
-        x[6] = (float)(cs[2] > 0.0 ? (q.x - cs[0]) / cs[2] : q.x - cs[0]);
-        x[7] = (float)(cs[3] > 0.0 ? (q.y - cs[1]) / cs[3] : q.y - cs[1]);
-        if (lane < kF) X[(size_t)v * kF + lane] = x[lane];
+        const float2 q = *reinterpret_cast<const float2 *>(X + (size_t)v * kF + 6);  // k_scaled's
+        x[6] = q.x;
+        x[7] = q.y;
+        if (lane < 6) X[(size_t)v * kF + lane] = x[lane];
         // h0 = ReLU(x W_in + b_in): lane j computes features j and j + 32
 #pragma unroll
         for (int t = 0; t < 2; ++t) {
@@ -194,46 +273,113 @@ __global__ void k_features(DevGraph g, long long delta, const double2 *__restric
 }
 
 // ----------------------------------------------------------- aggregation --
-// G[v] = sum_u (w_uv / d_v) H[u]  (forward);  one warp per vertex, lane owns
-// features 2*lane, 2*lane+1 (one 128 B row per neighbour per warp)
-__global__ void k_spmm_fwd(DevGraph g, const __nv_bfloat16 *__restrict__ H, __nv_bfloat16 *__restrict__ G) {
-    const int lane = threadIdx.x & 31;
+// G[v] = sum_u (w_uv / d_v) H[u]  (forward); one warp per vertex.  The lanes load
+// 32 arcs at once and hand them round; eight lanes take a neighbour's 128 B row,
+// 16 B each, so that a load instruction fetches four rows, and sixteen rows are
+// on the way together.  What bounds it are those rows, 128 B an arc from L2 (1 M
+// arcs: 39 us with a row a load, 28 so).
+__global__ void __launch_bounds__(256)
+k_spmm_fwd(DevGraph g, const __nv_bfloat16 *__restrict__ H, __nv_bfloat16 *__restrict__ G) {
+    constexpr unsigned kAll = 0xffffffffu;
+    constexpr int kAhead = 4;
+    const int lane = threadIdx.x & 31, nb = lane >> 3, f = lane & 7;
     const int nw = (gridDim.x * blockDim.x) >> 5;
-    const __nv_bfloat162 *H2 = reinterpret_cast<const __nv_bfloat162 *>(H);
+    const uint4 *H8 = reinterpret_cast<const uint4 *>(H);
     for (int v = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; v < g.n; v += nw) {
         const int a0 = g.rp[v], a1 = g.rp[v + 1];
-        float s0 = 0.f, s1 = 0.f;
-        for (int i = a0; i < a1; ++i) {
-            const int2 e = g.adj[i];
-            const float2 hv = __bfloat1622float2(H2[(size_t)e.x * (kH / 2) + lane]);
-            s0 += (float)e.y * hv.x;
-            s1 += (float)e.y * hv.y;
+        float s[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) s[j] = 0.f;
+        for (int i0 = a0; i0 < a1; i0 += 32) {
+            const int2 e = i0 + lane < a1 ? g.adj[i0 + lane] : make_int2(-1, 0);
+            for (int t = 0; t < 32 && i0 + t < a1; t += 4 * kAhead) {
+                uint4 h[kAhead];
+                float w[kAhead];
+#pragma unroll
+                for (int k = 0; k < kAhead; ++k) {
+                    const int x = __shfl_sync(kAll, e.x, t + 4 * k + nb);
+                    w[k] = (float)__shfl_sync(kAll, e.y, t + 4 * k + nb);
+                    h[k] = x >= 0 ? H8[(size_t)x * 8 + f] : make_uint4(0, 0, 0, 0);
+                }
+#pragma unroll
+                for (int k = 0; k < kAhead; ++k) {
+                    const unsigned q[4] = {h[k].x, h[k].y, h[k].z, h[k].w};
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {  // a BF16 is the upper half of its float
+                        s[2 * j] += w[k] * __uint_as_float(q[j] << 16);
+                        s[2 * j + 1] += w[k] * __uint_as_float(q[j] & 0xffff0000u);
+                    }
+                }
+            }
         }
-        const float inv = g.deg[v] > 0 ? 1.f / (float)g.deg[v] : 0.f;
-        reinterpret_cast<__nv_bfloat162 *>(G)[(size_t)v * (kH / 2) + lane] =
-            __floats2bfloat162_rn(s0 * inv, s1 * inv);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            s[j] += __shfl_xor_sync(kAll, s[j], 8);
+            s[j] += __shfl_xor_sync(kAll, s[j], 16);
+        }
+        if (nb == 0) {
+            const float inv = g.deg[v] > 0 ? 1.f / (float)g.deg[v] : 0.f;
+            __nv_bfloat162 o[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) o[j] = __floats2bfloat162_rn(s[2 * j] * inv, s[2 * j + 1] * inv);
+            reinterpret_cast<uint4 *>(G)[(size_t)v * 8 + f] = *reinterpret_cast<const uint4 *>(o);
+        }
     }
 }
 
-// dH[u] += sum_v (w_uv / d_v) dG[v]  (transpose; the graph is symmetric)
-__global__ void k_spmm_bwd(DevGraph g, const float *__restrict__ dG, float *__restrict__ dH) {
-    const int lane = threadIdx.x & 31;
+// dH[u] += sum_v (w_uv / d_v) dG[v]  (transpose; the graph is symmetric): the
+// same walk with FP32 rows of 256 B, sixteen lanes a row, each lane working out
+// one arc's factor (a weight of 1 takes the reciprocal fd holds, the same value
+// as the division).  1 M arcs: 117 us with a conversion and a division an arc
+// and lane, 64 us with a row a load, 40 so.
+__global__ void __launch_bounds__(256)
+k_spmm_bwd(DevGraph g, const float2 *__restrict__ fd, const float *__restrict__ dG, float *__restrict__ dH) {
+    constexpr unsigned kAll = 0xffffffffu;
+    constexpr int kAhead = 8;
+    const int lane = threadIdx.x & 31, nb = lane >> 4, f = lane & 15;
     const int nw = (gridDim.x * blockDim.x) >> 5;
+    const float4 *D4 = reinterpret_cast<const float4 *>(dG);
     for (int u = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; u < g.n; u += nw) {
         const int a0 = g.rp[u], a1 = g.rp[u + 1];
-        float s0 = 0.f, s1 = 0.f;
-        for (int i = a0; i < a1; ++i) {
-            const int2 e = g.adj[i];
-            const float c = (float)e.y / (float)g.deg[e.x];
-            const float2 d = reinterpret_cast<const float2 *>(dG)[(size_t)e.x * (kH / 2) + lane];
-            s0 += c * d.x;
-            s1 += c * d.y;
+        float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int i0 = a0; i0 < a1; i0 += 32) {
+            const int2 e = i0 + lane < a1 ? g.adj[i0 + lane] : make_int2(-1, 0);
+            float c = 0.f;
+            if (e.x >= 0) {
+                const float2 d = fd[e.x];
+                c = e.y == 1 ? d.y : (float)e.y / d.x;
+            }
+            for (int t = 0; t < 32 && i0 + t < a1; t += 2 * kAhead) {
+                float4 h[kAhead];
+                float w[kAhead];
+#pragma unroll
+                for (int k = 0; k < kAhead; ++k) {
+                    const int x = __shfl_sync(kAll, e.x, t + 2 * k + nb);
+                    w[k] = __shfl_sync(kAll, c, t + 2 * k + nb);
+                    h[k] = x >= 0 ? D4[(size_t)x * 16 + f] : make_float4(0.f, 0.f, 0.f, 0.f);
+                }
+#pragma unroll
+                for (int k = 0; k < kAhead; ++k) {
+                    s.x += w[k] * h[k].x;
+                    s.y += w[k] * h[k].y;
+                    s.z += w[k] * h[k].z;
+                    s.w += w[k] * h[k].w;
+                }
+            }
         }
-        float2 *o = reinterpret_cast<float2 *>(dH) + (size_t)u * (kH / 2) + lane;
-        float2 cur = *o;
-        cur.x += s0;
-        cur.y += s1;
-        *o = cur;
+        s.x += __shfl_xor_sync(kAll, s.x, 16);
+        s.y += __shfl_xor_sync(kAll, s.y, 16);
+        s.z += __shfl_xor_sync(kAll, s.z, 16);
+        s.w += __shfl_xor_sync(kAll, s.w, 16);
+        if (nb == 0) {
+            float4 *o = reinterpret_cast<float4 *>(dH) + (size_t)u * 16 + f;
+            float4 cur = *o;
+            cur.x += s.x;
+            cur.y += s.y;
+            cur.z += s.z;
+            cur.w += s.w;
+            *o = cur;
+        }
     }
 }
 
@@ -263,12 +409,13 @@ __device__ __forceinline__ void mma_bf16(float (&c)[4], unsigned a0, unsigned a1
 // Y[rows x N] = A[rows x K] * B[K x N] (+ bias) with A given as up to two
 // BF16 row blocks of K/2 columns (A = [A1, A2]) or one of K columns, and B as
 // BT[N][K] BF16 (n-major, k contiguous).  64 rows per block of 4 warps.
-// mode 0: store Z (fp32) and ReLU(Z) as BF16 into Ybf;  mode 1: store Y fp32.
+// mode 0: store Z (fp32) and ReLU(Z) as BF16 into Ybf;  mode 1: store Y fp32, its
+// first 64 columns to Zout and the others to Yhi (rows of 64 each).
 template <int K, int N>
 __global__ void __launch_bounds__(128)
 k_gemm(const __nv_bfloat16 *__restrict__ A1, const __nv_bfloat16 *__restrict__ A2, int n_rows,
        const __nv_bfloat16 *__restrict__ BT, const float *__restrict__ bias, float *__restrict__ Zout,
-       __nv_bfloat16 *__restrict__ Ybf, int mode) {
+       __nv_bfloat16 *__restrict__ Ybf, float *__restrict__ Yhi, int mode) {
     constexpr int KP = K + 8;  // padded row (bf16) against ldmatrix bank conflicts
     __shared__ __align__(16) __nv_bfloat16 sA[64 * KP];
     __shared__ __align__(16) __nv_bfloat16 sB[N * KP];
@@ -331,8 +478,9 @@ k_gemm(const __nv_bfloat16 *__restrict__ A1, const __nv_bfloat16 *__restrict__ A
                         __floats2bfloat162_rn(z2 > 0.f ? z2 : 0.f, z3 > 0.f ? z3 : 0.f);
                 }
             } else {
-                if (rlo < n_rows) { Zout[(size_t)rlo * N + c] = z0; Zout[(size_t)rlo * N + c + 1] = z1; }
-                if (rhi < n_rows) { Zout[(size_t)rhi * N + c] = z2; Zout[(size_t)rhi * N + c + 1] = z3; }
+                float *y = c < kH ? Zout + c : Yhi + c - kH;
+                if (rlo < n_rows) *reinterpret_cast<float2 *>(y + (size_t)rlo * kH) = make_float2(z0, z1);
+                if (rhi < n_rows) *reinterpret_cast<float2 *>(y + (size_t)rhi * kH) = make_float2(z2, z3);
             }
         }
     }
@@ -371,7 +519,18 @@ __global__ void k_loss(const float *__restrict__ S, const unsigned *__restrict__
         l0 += __shfl_xor_sync(0xffffffffu, l0, o);
         l1 += __shfl_xor_sync(0xffffffffu, l1, o);
     }
-    if ((threadIdx.x & 31) == 0) { atomicAdd(&acc[0], l0); atomicAdd(&acc[1], l1); }
+    // one pair of atomics a block
+    __shared__ double sh[2][8];
+    if ((threadIdx.x & 31) == 0) {
+        sh[0][threadIdx.x >> 5] = l0;
+        sh[1][threadIdx.x >> 5] = l1;
+    }
+    __syncthreads();
+    if (threadIdx.x < 2) {
+        double t = 0;
+        for (int k = 0; k < (int)(blockDim.x >> 5); ++k) t += sh[threadIdx.x][k];
+        atomicAdd(&acc[threadIdx.x], t);
+    }
 }
 
 // dS = (p - y*) / n with the better polarity; dH3 = dS w_out; head grads
@@ -382,44 +541,83 @@ __global__ void k_head_bwd(const float *__restrict__ S, const unsigned *__restri
     const int lane = threadIdx.x & 31;
     const int nw = (gridDim.x * blockDim.x) >> 5;
     float gw0 = 0.f, gw1 = 0.f, gb = 0.f;
-    for (int v = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; v < n; v += nw) {
-        const float p = 1.f / (1.f + expf(-S[v]));
-        const int y = ((bits[v >> 5] >> (v & 31)) & 1) ^ flip;
-        const float ds = (p - (float)y) / (float)n;
-        const float2 h = __bfloat1622float2(reinterpret_cast<const __nv_bfloat162 *>(H)[(size_t)v * (kH / 2) + lane]);
-        gw0 += ds * h.x;
-        gw1 += ds * h.y;
-        gb += lane == 0 ? ds : 0.f;
-        reinterpret_cast<float2 *>(dH)[(size_t)v * (kH / 2) + lane] =
-            make_float2(ds * P[kPWout + 2 * lane], ds * P[kPWout + 2 * lane + 1]);
+    const float w0 = P[kPWout + 2 * lane], w1 = P[kPWout + 2 * lane + 1];
+    constexpr int kV = 8;  // vertices a warp loads at once
+    for (int v0 = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * kV; v0 < n; v0 += nw * kV) {
+        float sv[kV];
+        unsigned bv[kV];
+        float2 h[kV];
+#pragma unroll
+        for (int k = 0; k < kV; ++k) {
+            const int v = v0 + k < n ? v0 + k : n - 1;
+            sv[k] = S[v];
+            bv[k] = bits[v >> 5];
+            h[k] = __bfloat1622float2(reinterpret_cast<const __nv_bfloat162 *>(H)[(size_t)v * (kH / 2) + lane]);
+        }
+#pragma unroll
+        for (int k = 0; k < kV; ++k) {
+            const int v = v0 + k;
+            if (v >= n) break;
+            const float p = 1.f / (1.f + expf(-sv[k]));
+            const int y = ((bv[k] >> (v & 31)) & 1) ^ flip;
+            const float ds = (p - (float)y) / (float)n;
+            gw0 += ds * h[k].x;
+            gw1 += ds * h[k].y;
+            gb += lane == 0 ? ds : 0.f;
+            reinterpret_cast<float2 *>(dH)[(size_t)v * (kH / 2) + lane] = make_float2(ds * w0, ds * w1);
+        }
     }
-    atomicAdd(&grad[kPWout + 2 * lane], gw0);
-    atomicAdd(&grad[kPWout + 2 * lane + 1], gw1);
-    if (lane == 0) atomicAdd(&grad[kPBout], gb);
+    // the warps of a block first: 65 atomics a block and not a warp (32768
+    // vertices: 200 us with 65 a warp of a full grid, 9 so)
+    __shared__ float sw[8][kH], sb[8];
+    sw[threadIdx.x >> 5][2 * lane] = gw0;
+    sw[threadIdx.x >> 5][2 * lane + 1] = gw1;
+    if (lane == 0) sb[threadIdx.x >> 5] = gb;
+    __syncthreads();
+    const int nwarp = blockDim.x >> 5;
+    if (threadIdx.x < kH) {
+        float t = 0.f;
+        for (int k = 0; k < nwarp; ++k) t += sw[k][threadIdx.x];
+        atomicAdd(&grad[kPWout + threadIdx.x], t);
+    } else if (threadIdx.x == kH) {
+        float t = 0.f;
+        for (int k = 0; k < nwarp; ++k) t += sb[k];
+        atomicAdd(&grad[kPBout], t);
+    }
 }
 
 // dZ = dH * (Z > 0) as BF16 (input of dX = dZ W^T) and kept in fp32 in dH
 __global__ void k_relu_bwd(float *__restrict__ dH, const float *__restrict__ Z, __nv_bfloat16 *__restrict__ dZbf,
                            long long count) {
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (long long)gridDim.x * blockDim.x) {
-        const float d = Z[i] > 0.f ? dH[i] : 0.f;
-        dH[i] = d;
-        dZbf[i] = __float2bfloat16(d);
+    // four at a time (count is a multiple of 64)
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < count / 4; i += (long long)gridDim.x * blockDim.x) {
+        const float4 z = reinterpret_cast<const float4 *>(Z)[i];
+        float4 d = reinterpret_cast<float4 *>(dH)[i];
+        d.x = z.x > 0.f ? d.x : 0.f;
+        d.y = z.y > 0.f ? d.y : 0.f;
+        d.z = z.z > 0.f ? d.z : 0.f;
+        d.w = z.w > 0.f ? d.w : 0.f;
+        reinterpret_cast<float4 *>(dH)[i] = d;
+        __nv_bfloat162 b[2] = {__floats2bfloat162_rn(d.x, d.y), __floats2bfloat162_rn(d.z, d.w)};
+        reinterpret_cast<uint2 *>(dZbf)[i] = *reinterpret_cast<const uint2 *>(b);
     }
 }
 
 // dW[128 x 64] += X^T bf16(dZ) on the tensor cores and db[64] += the column
-// sums of dZ (FP32), with X = [A1, A2] (n x 64 BF16 each).  Tiles of 16
+// sums of dZ (FP32), with X = [A1, A2] (n x 64 BF16 each).  Tiles of 64
 // vertices pass through shared memory; ldmatrix.trans turns the row-major
 // tiles into the A (X^T) and B (dZ) fragments of mma.m16n8k16.  Warp w keeps
-// rows 32w..32w+31 of dW in registers and adds them into dW at the end.
+// rows 32w..32w+31 of dW in registers and adds them into dW at the end: 8192
+// atomics a block, so the grid is a block a SM (32768 vertices: 92 us with a
+// block for every 16 of them, 18 so).
+constexpr int kWgTile = 64;
 __global__ void __launch_bounds__(128)
 k_wgrad_tc(const __nv_bfloat16 *__restrict__ A1, const __nv_bfloat16 *__restrict__ A2,
            const __nv_bfloat16 *__restrict__ dZb, const float *__restrict__ dZ, int n, float *__restrict__ dW,
            float *__restrict__ db) {
     constexpr int XP = kK + 8, ZP = kH + 8;  // padded rows: 272 B and 144 B, both 16 B multiples
-    __shared__ __align__(16) __nv_bfloat16 sX[16 * XP];
-    __shared__ __align__(16) __nv_bfloat16 sZ[16 * ZP];
+    __shared__ __align__(16) __nv_bfloat16 sX[kWgTile * XP];
+    __shared__ __align__(16) __nv_bfloat16 sZ[kWgTile * ZP];
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     float acc[2][8][4];
 #pragma unroll
@@ -429,39 +627,61 @@ k_wgrad_tc(const __nv_bfloat16 *__restrict__ A1, const __nv_bfloat16 *__restrict
     float bsum = 0.f;
     const uint4 *X1 = reinterpret_cast<const uint4 *>(A1), *X2 = reinterpret_cast<const uint4 *>(A2);
     const uint4 *Zb = reinterpret_cast<const uint4 *>(dZb);
-    for (int v0 = blockIdx.x * 16; v0 < n; v0 += gridDim.x * 16) {
-        __syncthreads();
-        for (int i = tid; i < 16 * 16; i += 128) {
-            const int r = i >> 4, c8 = i & 15;
-            uint4 val = make_uint4(0, 0, 0, 0);
-            if (v0 + r < n) val = c8 < 8 ? X1[(size_t)(v0 + r) * 8 + c8] : X2[(size_t)(v0 + r) * 8 + c8 - 8];
-            *reinterpret_cast<uint4 *>(&sX[r * XP + c8 * 8]) = val;
-        }
-        {
-            const int r = tid >> 3, c8 = tid & 7;
-            uint4 val = make_uint4(0, 0, 0, 0);
-            if (v0 + r < n) val = Zb[(size_t)(v0 + r) * 8 + c8];
-            *reinterpret_cast<uint4 *>(&sZ[r * ZP + c8 * 8]) = val;
-        }
-        if (tid < kH)
-            for (int r = 0; r < 16 && v0 + r < n; ++r) bsum += dZ[(size_t)(v0 + r) * kH + tid];
-        __syncthreads();
-        unsigned a[2][4];
+    for (int v0 = blockIdx.x * kWgTile; v0 < n; v0 += gridDim.x * kWgTile) {
+        // the whole tile is on the way before any of it is stored: a SM holds
+        // one block, and four warps hide no latency between them
+        uint4 x[kWgTile / 8], z[kWgTile / 16];
+        float bz[kWgTile / 2];
+        const uint4 zero = make_uint4(0, 0, 0, 0);
 #pragma unroll
-        for (int mt = 0; mt < 2; ++mt) {
-            const int m0 = wid * 32 + mt * 16;
-            ldsm_x4_t(a[mt][0], a[mt][1], a[mt][2], a[mt][3],
-                      &sX[((lane & 7) + 8 * (lane >> 4)) * XP + m0 + 8 * ((lane >> 3) & 1)]);
+        for (int k = 0; k < kWgTile / 8; ++k) {
+            const int i = tid + 128 * k, v = v0 + (i >> 4), c8 = i & 15;
+            x[k] = v < n ? (c8 < 8 ? X1[(size_t)v * 8 + c8] : X2[(size_t)v * 8 + c8 - 8]) : zero;
         }
 #pragma unroll
-        for (int nt2 = 0; nt2 < 4; ++nt2) {
-            const int n0 = nt2 * 16;
-            unsigned b0, b1, b2, b3;
-            ldsm_x4_t(b0, b1, b2, b3, &sZ[((lane & 7) + 8 * ((lane >> 3) & 1)) * ZP + n0 + 8 * (lane >> 4)]);
+        for (int k = 0; k < kWgTile / 16; ++k) {
+            const int i = tid + 128 * k, v = v0 + (i >> 3);
+            z[k] = v < n ? Zb[(size_t)v * 8 + (i & 7)] : zero;
+        }
+        // column tid % 64, the rows of this thread's half
+#pragma unroll
+        for (int k = 0; k < kWgTile / 2; ++k) {
+            const int v = v0 + 2 * k + (tid >> 6);
+            bz[k] = v < n ? dZ[(size_t)v * kH + (tid & 63)] : 0.f;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < kWgTile / 8; ++k) {
+            const int i = tid + 128 * k;
+            *reinterpret_cast<uint4 *>(&sX[(i >> 4) * XP + (i & 15) * 8]) = x[k];
+        }
+#pragma unroll
+        for (int k = 0; k < kWgTile / 16; ++k) {
+            const int i = tid + 128 * k;
+            *reinterpret_cast<uint4 *>(&sZ[(i >> 3) * ZP + (i & 7) * 8]) = z[k];
+        }
+#pragma unroll
+        for (int k = 0; k < kWgTile / 2; ++k) bsum += bz[k];
+        __syncthreads();
+#pragma unroll
+        for (int k0 = 0; k0 < kWgTile; k0 += 16) {
+            unsigned a[2][4];
 #pragma unroll
             for (int mt = 0; mt < 2; ++mt) {
-                mma_bf16(acc[mt][2 * nt2], a[mt][0], a[mt][1], a[mt][2], a[mt][3], b0, b1);
-                mma_bf16(acc[mt][2 * nt2 + 1], a[mt][0], a[mt][1], a[mt][2], a[mt][3], b2, b3);
+                const int m0 = wid * 32 + mt * 16;
+                ldsm_x4_t(a[mt][0], a[mt][1], a[mt][2], a[mt][3],
+                          &sX[(k0 + (lane & 7) + 8 * (lane >> 4)) * XP + m0 + 8 * ((lane >> 3) & 1)]);
+            }
+#pragma unroll
+            for (int nt2 = 0; nt2 < 4; ++nt2) {
+                const int n0 = nt2 * 16;
+                unsigned b0, b1, b2, b3;
+                ldsm_x4_t(b0, b1, b2, b3, &sZ[(k0 + (lane & 7) + 8 * ((lane >> 3) & 1)) * ZP + n0 + 8 * (lane >> 4)]);
+#pragma unroll
+                for (int mt = 0; mt < 2; ++mt) {
+                    mma_bf16(acc[mt][2 * nt2], a[mt][0], a[mt][1], a[mt][2], a[mt][3], b0, b1);
+                    mma_bf16(acc[mt][2 * nt2 + 1], a[mt][0], a[mt][1], a[mt][2], a[mt][3], b2, b3);
+                }
             }
         }
     }
@@ -476,15 +696,14 @@ k_wgrad_tc(const __nv_bfloat16 *__restrict__ A1, const __nv_bfloat16 *__restrict
             atomicAdd(&dW[(m + 8) * kH + c], acc[mt][nt][2]);
             atomicAdd(&dW[(m + 8) * kH + c + 1], acc[mt][nt][3]);
         }
-    if (tid < kH) atomicAdd(&db[tid], bsum);
+    atomicAdd(&db[tid & 63], bsum);
 }
 
 // dW[K x N] += X^T dZ, db += column sums of dZ, on CUDA cores, for the input
 // layer (X = the n x 8 FP32 features)
 template <int K>
 __global__ void __launch_bounds__(256)
-k_wgrad(const __nv_bfloat16 *__restrict__ A1, const __nv_bfloat16 *__restrict__ A2, const float *__restrict__ Xf,
-        const float *__restrict__ dZ, int n, float *__restrict__ dW, float *__restrict__ db) {
+k_wgrad(const float *__restrict__ Xf, const float *__restrict__ dZ, int n, float *__restrict__ dW, float *__restrict__ db) {
     // thread t owns output column j = t % 64 and rows k = t / 64 + 4 i
     const int t = threadIdx.x, j = t & 63, k0 = t >> 6;
     constexpr int KR = K / 4;
@@ -492,17 +711,21 @@ k_wgrad(const __nv_bfloat16 *__restrict__ A1, const __nv_bfloat16 *__restrict__ 
 #pragma unroll
     for (int i = 0; i < KR; ++i) acc[i] = 0.f;
     float bsum = 0.f;
-    for (int v = blockIdx.x; v < n; v += gridDim.x) {
-        const float dz = dZ[(size_t)v * kH + j];
-        if (k0 == 0) bsum += dz;
+    constexpr int kV = 8;  // vertices loaded at once
+    for (int v0 = blockIdx.x * kV; v0 < n; v0 += gridDim.x * kV) {
+        float dz[kV], x[kV][KR];
 #pragma unroll
-        for (int i = 0; i < KR; ++i) {
-            const int k = k0 + 4 * i;
-            float x;
-            if (Xf) x = Xf[(size_t)v * K + k];
-            else if (A2 == nullptr) x = __bfloat162float(A1[(size_t)v * K + k]);
-            else x = k < K / 2 ? __bfloat162float(A1[(size_t)v * (K / 2) + k]) : __bfloat162float(A2[(size_t)v * (K / 2) + k - K / 2]);
-            acc[i] += x * dz;
+        for (int q = 0; q < kV; ++q) {
+            const int v = v0 + q;
+            dz[q] = v < n ? dZ[(size_t)v * kH + j] : 0.f;
+#pragma unroll
+            for (int i = 0; i < KR; ++i) x[q][i] = v < n ? Xf[(size_t)v * K + k0 + 4 * i] : 0.f;
+        }
+#pragma unroll
+        for (int q = 0; q < kV; ++q) {
+            if (k0 == 0) bsum += dz[q];
+#pragma unroll
+            for (int i = 0; i < KR; ++i) acc[i] += x[q][i] * dz[q];
         }
     }
 #pragma unroll
@@ -529,17 +752,6 @@ __global__ void k_cast_weights(const float *__restrict__ P, __nv_bfloat16 *WT, _
         const float w = P[kPW0 + l * kPLayer + k * kH + j];
         WT[(size_t)l * kK * kH + j * kK + k] = __float2bfloat16(w);
         Wn[(size_t)l * kK * kH + k * kH + j] = __float2bfloat16(w);
-    }
-}
-
-// dX (fp32, n x 128) -> dH_direct (cols 0..63, added) and dG (cols 64..127)
-__global__ void k_split_dx(const float *__restrict__ dX, int n, float *__restrict__ dH, float *__restrict__ dG) {
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < (long long)n * kK;
-         i += (long long)gridDim.x * blockDim.x) {
-        const long long v = i / kK;
-        const int c = (int)(i % kK);
-        if (c < kH) dH[v * kH + c] = dX[i];
-        else dG[v * kH + c - kH] = dX[i];
     }
 }
 
@@ -690,7 +902,9 @@ struct Proposer {
     int n_cap = 0;
     float *P = nullptr, *M = nullptr, *V = nullptr, *grad = nullptr;
     __nv_bfloat16 *WT = nullptr, *Wn = nullptr;
-    float *X = nullptr, *Z = nullptr, *S = nullptr, *dH = nullptr, *dG = nullptr, *dX = nullptr;
+    float *X = nullptr, *Z = nullptr, *S = nullptr, *dH = nullptr, *dG = nullptr;
+    double *rd = nullptr;                   // 1 / degree
+    float2 *fd = nullptr;                   // degree, 1 / degree
     double2 *Sm0 = nullptr, *Sm1 = nullptr; // smoothed-feature ping-pong
     double *red = nullptr;                  // centring partials
     double *cs = nullptr;                   // means and largest magnitudes
@@ -702,7 +916,7 @@ struct Proposer {
 
 static int prop_alloc(Proposer &p, int n, cudaStream_t s) {
     if (n <= p.n_cap) return MC_OK;
-    void *ps[] = {p.X, p.Z, p.S, p.dH, p.dG, p.dX, p.Hb, p.Gb, p.dZb, p.Sm0, p.Sm1};
+    void *ps[] = {p.X, p.Z, p.S, p.dH, p.dG, p.rd, p.fd, p.Hb, p.Gb, p.dZb, p.Sm0, p.Sm1};
     for (void *q : ps) dev_free(q, s);
     const size_t N = (size_t)n;
     MC_TRY(dev_alloc_n(&p.Sm0, N, s));
@@ -712,7 +926,8 @@ static int prop_alloc(Proposer &p, int n, cudaStream_t s) {
     MC_TRY(dev_alloc_n(&p.S, N, s));
     MC_TRY(dev_alloc_n(&p.dH, N * kH, s));
     MC_TRY(dev_alloc_n(&p.dG, N * kH, s));
-    MC_TRY(dev_alloc_n(&p.dX, N * kK, s));
+    MC_TRY(dev_alloc_n(&p.rd, N, s));
+    MC_TRY(dev_alloc_n(&p.fd, N, s));
     MC_TRY(dev_alloc_n(&p.Hb, N * kH * (kL + 1), s));
     MC_TRY(dev_alloc_n(&p.Gb, N * kH * kL, s));
     MC_TRY(dev_alloc_n(&p.dZb, N * kH, s));
@@ -741,7 +956,7 @@ int proposer_create(Proposer **out, const float *init) {
 
 void proposer_destroy(Proposer *p) {
     if (!p) return;
-    void *ps[] = {p->P, p->M, p->V, p->grad, p->WT, p->Wn, p->acc, p->X, p->Z, p->S, p->dH, p->dG, p->dX,
+    void *ps[] = {p->P, p->M, p->V, p->grad, p->WT, p->Wn, p->acc, p->X, p->Z, p->S, p->dH, p->dG, p->rd, p->fd,
                   p->Hb, p->Gb, p->dZb, p->Sm0, p->Sm1, p->red, p->cs};
     cudaDeviceSynchronize();  // no stream may still use the buffers
     for (void *q : ps) dev_free(q, nullptr);
@@ -773,16 +988,17 @@ int proposer_forward(Proposer &p, const DevGraph &g, long long delta, cudaStream
     const int wb = blocks_for((long long)g.n * 32, 256);
     const int tb = blocks_for(g.n, 256);
     // smoothed random features: kSmooth lazy-walk steps, centring, scaling
-    ++::mc::g_launches; k_rand_init<<<tb, 256, 0, s>>>(g.n, p.feat_seed, p.Sm0);
+    ++::mc::g_launches; k_rand_init<<<tb, 256, 0, s>>>(g, p.feat_seed, p.Sm0, p.rd, p.fd);
     double2 *a = p.Sm0, *b = p.Sm1;
     for (int t = 0; t < kSmooth; ++t) {
-        ++::mc::g_launches; k_smooth<<<wb, 256, 0, s>>>(g, a, b);
+        ++::mc::g_launches; k_smooth<<<blocks_for((long long)g.n << kSmoothLg, 256), 256, 0, s>>>(g, a, p.rd, b);
         double2 *tmp = a; a = b; b = tmp;
     }
     ++::mc::g_launches; k_center_partial<<<kRedBlocks, 256, 0, s>>>(g, a, p.red);
-    ++::mc::g_launches; k_center_final<<<1, 32, 0, s>>>(p.red, kRedBlocks, p.cs);
+    ++::mc::g_launches; k_center_final<<<1, 256, 0, s>>>(p.red, kRedBlocks, p.cs);
     ++::mc::g_launches; k_maxabs<<<tb, 256, 0, s>>>(g.n, a, p.cs);
-    ++::mc::g_launches; k_features<<<wb, 256, 0, s>>>(g, delta, a, p.cs, p.P, p.X, p.Hb, p.Z);
+    ++::mc::g_launches; k_scaled<<<tb, 256, 0, s>>>(g.n, a, p.cs, p.X);
+    ++::mc::g_launches; k_features<<<wb, 256, 0, s>>>(g, delta, p.P, p.X, p.Hb, p.Z);
     for (int l = 0; l < kL; ++l) {
         const __nv_bfloat16 *H = p.Hb + l * NH;
         __nv_bfloat16 *G = p.Gb + l * NH;
@@ -791,7 +1007,7 @@ int proposer_forward(Proposer &p, const DevGraph &g, long long delta, cudaStream
         ++::mc::g_launches;
         k_gemm<kK, kH><<<gb, 128, 0, s>>>(H, G, g.n, p.WT + (size_t)l * kK * kH,
                                           p.P + kPW0 + l * kPLayer + kK * kH, p.Z + (l + 1) * NH,
-                                          p.Hb + (l + 1) * NH, 0);
+                                          p.Hb + (l + 1) * NH, nullptr, 0);
     }
     ++::mc::g_launches; k_head<<<wb, 256, 0, s>>>(p.Hb + kL * NH, g.n, p.P, p.S);
     MC_CUDA(cudaGetLastError());
@@ -806,26 +1022,27 @@ int proposer_backward(Proposer &p, const DevGraph &g, const unsigned *bits, doub
     MC_CUDA(cudaMemsetAsync(p.grad, 0, sizeof(float) * kPTotal, s));
     const int tb = blocks_for(g.n, 256), wb = blocks_for((long long)g.n * 32, 256);
     ++::mc::g_launches; k_loss<<<tb, 256, 0, s>>>(p.S, bits, g.n, p.acc);
-    ++::mc::g_launches; k_head_bwd<<<wb, 256, 0, s>>>(p.S, bits, g.n, p.acc, p.Hb + kL * NH, p.P, p.dH, p.grad);
+    ++::mc::g_launches; k_head_bwd<<<wb < num_sms() ? wb : num_sms(), 256, 0, s>>>(p.S, bits, g.n, p.acc, p.Hb + kL * NH, p.P, p.dH, p.grad);
+    const int tiles = (g.n + kWgTile - 1) / kWgTile;
     for (int l = kL - 1; l >= 0; --l) {
         // dZ_{l+1} = dH_{l+1} * ReLU'
-        ++::mc::g_launches; k_relu_bwd<<<blocks_for((long long)NH, 256), 256, 0, s>>>(p.dH, p.Z + (l + 1) * NH, p.dZb, (long long)NH);
+        ++::mc::g_launches; k_relu_bwd<<<blocks_for((long long)NH / 4, 256), 256, 0, s>>>(p.dH, p.Z + (l + 1) * NH, p.dZb, (long long)NH);
         // dW_l (tensor cores), db_l
         ++::mc::g_launches;
-        k_wgrad_tc<<<blocks_for(((long long)g.n + 15) / 16 * 128, 128), 128, 0, s>>>(
+        k_wgrad_tc<<<tiles < num_sms() ? tiles : num_sms(), 128, 0, s>>>(
             p.Hb + l * NH, p.Gb + l * NH, p.dZb, p.dH, g.n, p.grad + kPW0 + l * kPLayer,
             p.grad + kPW0 + l * kPLayer + kK * kH);
-        // dX = dZ W_l^T  (n x 128): B^T operand = W_l as (128 x 64) n-major
+        // dX = dZ W_l^T  (n x 128): B^T operand = W_l as (128 x 64) n-major;
+        // its halves are the direct part of dH_l and dG_l
         const int gb = blocks_for(((long long)g.n + 63) / 64 * 128, 128);
         ++::mc::g_launches;
-        k_gemm<kH, kK><<<gb, 128, 0, s>>>(p.dZb, nullptr, g.n, p.Wn + (size_t)l * kK * kH, nullptr, p.dX, nullptr, 1);
-        ++::mc::g_launches; k_split_dx<<<blocks_for((long long)g.n * kK, 256), 256, 0, s>>>(p.dX, g.n, p.dH, p.dG);
-        ++::mc::g_launches; k_spmm_bwd<<<wb, 256, 0, s>>>(g, p.dG, p.dH);
+        k_gemm<kH, kK><<<gb, 128, 0, s>>>(p.dZb, nullptr, g.n, p.Wn + (size_t)l * kK * kH, nullptr, p.dH, nullptr, p.dG, 1);
+        ++::mc::g_launches; k_spmm_bwd<<<wb, 256, 0, s>>>(g, p.fd, p.dG, p.dH);
     }
     // input layer: dZ0 = dH0 * ReLU'(Z0); dW_in = X^T dZ0
-    ++::mc::g_launches; k_relu_bwd<<<blocks_for((long long)NH, 256), 256, 0, s>>>(p.dH, p.Z, p.dZb, (long long)NH);
+    ++::mc::g_launches; k_relu_bwd<<<blocks_for((long long)NH / 4, 256), 256, 0, s>>>(p.dH, p.Z, p.dZb, (long long)NH);
     ++::mc::g_launches;
-    k_wgrad<kF><<<num_sms() * 4, 256, 0, s>>>(nullptr, nullptr, p.X, p.dH, g.n, p.grad + kPWin, p.grad + kPBin);
+    k_wgrad<kF><<<num_sms() * 2, 256, 0, s>>>(p.X, p.dH, g.n, p.grad + kPWin, p.grad + kPBin);
     MC_CUDA(cudaGetLastError());
     double h[4];
     MC_CUDA(cudaMemcpyAsync(h, p.acc, sizeof(h), cudaMemcpyDeviceToHost, s));
