@@ -332,10 +332,13 @@ k_emit_half(const int *__restrict__ src, const int2 *__restrict__ adj, i64 arcs,
             bool first = cross;
             if (merge) {
                 const unsigned peers = __match_any_sync(kAll, cross ? key : ~(u64)lane);
-                if (cross) {
+                first = cross && lane == __ffs(peers) - 1;
+                if (__all_sync(kAll, !cross || c == 1)) {
+                    c = __popc(peers);
+                    c = c < cap ? c : cap;
+                } else if (cross) {  // a reduction for each distinct key
                     const unsigned sum = __reduce_add_sync(peers, (unsigned)c);
                     c = sum < (unsigned)cap ? (int)sum : cap;
-                    first = lane == __ffs(peers) - 1;
                 }
             }
             out.room(64);
