@@ -207,14 +207,18 @@ int mc_min_cut(mc_graph *g, const mc_options *opt, int64_t *lambda_out,
  *   bitmaps   NULL, or per-graph side bitmaps: graph g's ceil(n_g/32) words
  *             start at bitmap_word_off[g] (host)
  *   bitmap_word_off  G+1 int64, required when bitmaps is non-NULL
- * One kernel launch solves the whole batch: one warp per graph, graphs
+ * With no shape chosen (mc_batch_set_shape, mc_batch_autotune) and the default
+ * queue order, canonical graphs of up to 2048 vertices whose state fits in
+ * shared memory are solved one block per graph, by rounds of forest packing
+ * and a dense finish.  The others (a batch mostly of several hundred graphs of
+ * 33 to 95 vertices among them), and all of them under a chosen shape, go to one launch with a warp per graph, graphs
  * taken largest first (Alg. 2 per graph with full capped scans, PR1/PR2 when
  * opt->pr_level >= 1 and the kernel shape in use runs them, and
  * in-warp contraction).  Self-loops and zero weights are dropped and
  * parallel arcs merged; after that every graph must be symmetric (each arc
  * (u, v, c) has its mirror (v, u, c)), which the kernel checks per graph; a
  * disconnected graph gets lambda 0.  stats: n_input/m_input are totals,
- * ms_total is the kernel's device time.
+ * ms_total is the kernels' device time.
  * Errors: MC_EINVAL (n_g < 2, bad offsets -- a graph's first offset not 0 or
  * its last not its arc count, refused before any launch, or an offset below
  * its predecessor, found by the kernel before it reads that graph's arcs --,

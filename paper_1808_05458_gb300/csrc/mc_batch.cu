@@ -22,6 +22,7 @@
 #include <vector>
 
 #include "mc_internal.cuh"
+#include "mc_batch_cta.cuh"
 #include "mc_scan.cuh"
 
 namespace mc {
@@ -121,6 +122,7 @@ struct BatchIn {
     const long long *voff, *aoff;
     const int *rp, *col, *w;
     const int *order;  // graphs, largest first
+    const int *count;  // how many of them; null: all G
     long long *lam_out;
     u32 *bits_out;                // may be null
     const long long *bits_off;    // word offsets, may be null
@@ -1318,11 +1320,12 @@ __global__ void __launch_bounds__(WPB * 32) k_batch(BatchIn B) {
     const int wid = threadIdx.x >> 5;
     const int gw = blockIdx.x * WPB + wid;
     Scratch S0 = scratch_of(B.scratch + (size_t)gw * B.L.bytes, B.L);
+    const int G = B.count ? *B.count : B.G;
     while (true) {
         int k = 0;
         if (lane_id() == 0) k = atomicAdd(B.next, 1);
         k = __shfl_sync(0xffffffffu, k, 0);
-        if (k >= B.G) break;
+        if (k >= G) break;
         solve_one<SN>(B, B.order[k], S0, smem[wid]);
     }
 }
@@ -1378,7 +1381,7 @@ struct BatchCtx {
     // batch layout; replayed while the layout (and so every kernel
     // argument) is unchanged
     cudaGraphExec_t exec = nullptr;
-    unsigned char key[sizeof(BatchIn) + 3 * sizeof(int)] = {};
+    unsigned char key[sizeof(BatchIn) + 8 * sizeof(int)] = {};
     long long replays = 0;
 };
 std::mutex g_batch_mutex;
@@ -1489,6 +1492,41 @@ int batch_solve(int G, const long long *vtx_off, const long long *arc_off, const
     if (shape < 0) shape = g_shape_choice;
     const bool tuned = shape >= 0;
     if (!tuned) shape = default_shape(G, nmax);
+    // a batch nobody tuned goes to the block-per-graph solver first, and what
+    // that leaves, or is not meant for it, to this one; a pinned or tuned shape
+    // is this one's alone.  `order` then holds the first solver's graphs by
+    // class, largest first, and behind them this one's
+    //
+    // Many graphs of 33 to 95 vertices and little else stay with the warps: the
+    // matrix's one chain takes the time there, and a SM runs sixteen and more of
+    // the warps' chains at once against four.  1216 graphs, weights to 100: 60
+    // vertices 0.19 ms a warp each, 0.24 a block; 120: 0.33 and 0.31; 400: 0.92
+    // and 0.36; 30: 0.20 and 0.07.  Few of them among others are the blocks'
+    // (96 graphs of 50 to 400: 0.36 ms with those below 96 behind the rest, 0.16).
+    const bool cta = !tuned && o.pq_order != MC_PQ_FIFO;
+    int chains = 0;
+    for (int k = 0; k < G; ++k) chains += batch_cta_chain((int)(vtx_off[k + 1] - vtx_off[k]));
+    const bool chains_warps = chains > G / 2 && chains > 4 * num_sms();
+    int cls_first[kCtaClasses + 1] = {}, n_cta = 0;
+    if (cta) {
+        std::vector<int> by[kCtaClasses + 1];
+        for (const int k : order) {
+            const int n = (int)(vtx_off[k + 1] - vtx_off[k]);
+            const int c = chains_warps && batch_cta_chain(n) ? -1 : batch_cta_class(n, arc_off[k + 1] - arc_off[k]);
+            by[c < 0 ? kCtaClasses : c].push_back(k);
+        }
+        order.clear();
+        for (int c = 0; c <= kCtaClasses; ++c) {
+            cls_first[c] = n_cta;
+            if (c < kCtaClasses) n_cta += (int)by[c].size();
+            order.insert(order.end(), by[c].begin(), by[c].end());
+        }
+    }
+    // the counters: the warps' next graph; each class's; the graphs in the rest
+    // list, which grows behind those it starts with
+    order.resize(2 * (size_t)G);
+    order.insert(order.end(), {0, 0, 0, 0, G - n_cta});
+    static_assert(kCtaClasses == 3, "one counter a class");
     const Layout L = make_layout(nmax, amax);
     const int wpb = kShapes[shape].wpb;
     const int warps_res = blocks_per_sm(shape) * wpb * num_sms();
@@ -1502,8 +1540,8 @@ int batch_solve(int G, const long long *vtx_off, const long long *arc_off, const
     auto take = [&](size_t bytes) { size_t r = off; off += al(bytes); return r; };
     const size_t o_voff = take(8 * (G + 1)), o_aoff = take(8 * (G + 1)), o_rp = take(4 * (V + G)),
                  o_col = take(4 * (A > 0 ? A : 1)), o_w = take(4 * (A > 0 ? A : 1)),
-                 o_ord = take(4 * G), o_lam = take(8 * G), o_err = take(4 * G),
-                 o_bits = take(4 * (bw > 0 ? bw : 1)), o_boff = take(8 * (G + 1)), o_next = take(4);
+                 o_ord = take(4 * order.size()), o_lam = take(8 * G), o_err = take(4 * G),
+                 o_bits = take(4 * (bw > 0 ? bw : 1)), o_boff = take(8 * (G + 1));
     MC_TRY(grow(&ctx.io, &ctx.io_bytes, off, s));
     MC_TRY(grow(reinterpret_cast<void **>(&ctx.scratch), &ctx.scratch_bytes, L.bytes * (size_t)warps, s));
     unsigned char *io = static_cast<unsigned char *>(ctx.io);
@@ -1514,7 +1552,7 @@ int batch_solve(int G, const long long *vtx_off, const long long *arc_off, const
         MC_CUDA(cudaMemcpyAsync(io + o_col, col, 4 * A, cudaMemcpyHostToDevice, s));
         MC_CUDA(cudaMemcpyAsync(io + o_w, w, 4 * A, cudaMemcpyHostToDevice, s));
     }
-    MC_CUDA(cudaMemcpyAsync(io + o_ord, order.data(), 4 * (size_t)G, cudaMemcpyHostToDevice, s));
+    MC_CUDA(cudaMemcpyAsync(io + o_ord, order.data(), 4 * order.size(), cudaMemcpyHostToDevice, s));
     if (bitmaps) MC_CUDA(cudaMemcpyAsync(io + o_boff, bitmap_word_off, 8 * (G + 1), cudaMemcpyHostToDevice, s));
 
 
@@ -1531,14 +1569,38 @@ int batch_solve(int G, const long long *vtx_off, const long long *arc_off, const
     B.err_out = (int *)(io + o_err);
     B.bits_out = bitmaps ? (u32 *)(io + o_bits) : nullptr;
     B.bits_off = bitmaps ? (const long long *)(io + o_boff) : nullptr;
-    B.next = (int *)(io + o_next);
+    B.next = (int *)(io + o_ord) + 2 * (size_t)G;
     B.scratch = ctx.scratch;
     B.L = L;
     B.seed = o.seed;
     B.pr_level = kShapes[shape].pr ? o.pr_level : 0;
-    B.pr_late = !tuned;
     B.fifo = o.pq_order == MC_PQ_FIFO;
-
+    B.pr_late = !tuned;
+    CtaBatch C;
+    memset(&C, 0, sizeof(C));
+    if (cta) {
+        C.voff = B.voff;
+        C.aoff = B.aoff;
+        C.rp = B.rp;
+        C.col = B.col;
+        C.w = B.w;
+        C.order = B.order;
+        C.lam_out = B.lam_out;
+        C.bits_out = B.bits_out;
+        C.bits_off = B.bits_off;
+        C.err_out = B.err_out;
+        C.next = B.next + 1;
+        C.nrest = B.next + 1 + kCtaClasses;
+        C.rest = (int *)(io + o_ord) + n_cta;
+        for (int c = 0; c < kCtaClasses; ++c) {
+            C.first[c] = cls_first[c];
+            C.count[c] = cls_first[c + 1] - cls_first[c];
+        }
+        C.seed = o.seed;
+        C.pr_level = o.pr_level;
+        B.order = C.rest;
+        B.count = C.nrest;
+    }
     cudaEvent_t ea, eb;
     cudaEventCreate(&ea);
     cudaEventCreate(&eb);
@@ -1548,19 +1610,21 @@ int batch_solve(int G, const long long *vtx_off, const long long *arc_off, const
     {
         unsigned char key[sizeof(ctx.key)];
         memcpy(key, &B, sizeof(BatchIn));
-        const int extra[3] = {shape, warps, (int)(o.cuda_stream != nullptr)};
+        // (the block-per-graph launch follows from B and the same choices)
+        const int extra[] = {shape, warps, (int)(o.cuda_stream != nullptr), (int)cta, o.pr_level,
+                             cls_first[1], cls_first[2], cls_first[3]};
         memcpy(key + sizeof(BatchIn), extra, sizeof(extra));
         if (!ctx.exec || memcmp(key, ctx.key, sizeof(key)) != 0) {
             if (ctx.exec) { cudaGraphExecDestroy(ctx.exec); ctx.exec = nullptr; }
             cudaGraph_t graph = nullptr;
             MC_CUDA(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
-            cudaError_t ce = cudaMemsetAsync(io + o_next, 0, 4, s);
-            if (ce == cudaSuccess) rc = run_batch(shape, B, warps, s);
+            if (cta) rc = batch_cta_launch(C, s);
+            if (rc == MC_OK) rc = run_batch(shape, B, warps, s);
             cudaError_t ee = cudaStreamEndCapture(s, &graph);
-            if (ce != cudaSuccess || ee != cudaSuccess || rc != MC_OK) {
+            if (ee != cudaSuccess || rc != MC_OK) {
                 if (graph) cudaGraphDestroy(graph);
                 if (rc != MC_OK) return rc;
-                set_cuda_error(ce != cudaSuccess ? ce : ee, "batch graph capture");
+                set_cuda_error(ee, "batch graph capture");
                 return MC_ECUDA;
             }
             cudaError_t ie = cudaGraphInstantiate(&ctx.exec, graph, 0);

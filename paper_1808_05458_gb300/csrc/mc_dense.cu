@@ -1,328 +1,36 @@
-// mc_dense.cu -- the last rounds of Alg. 2 on a dense matrix in shared memory.
-//
-// A contracted graph of at most 224 vertices fits one block's shared memory as
-// a matrix of 32-bit weights (clamped at the bound as everywhere).  One warp
-// then scans it (Alg. 3): a lane owns every 32nd column -- its r-value and join
-// in registers -- so that a pop is a load of the popped row, an update a column
-// and one warp maximum over (key, vertex) words, with no queue and no list of
-// arcs.  The whole block does what surrounds the scan: PR1/PR2 and the degree-2
-// rule, the unions, the contraction (rows added up in place, a thread a column,
-// then columns, a warp a row) and the degrees.
-//
-// The rounds, their start vertices, the order of pops (the smallest vertex of
-// the largest key) and so every result are those of the single-warp solver
-// over lists (mc_batch.cu, k_tail), which larger graphs and bounds keep.
-// Bound by the scan's chain of dependent instructions: about 370 cycles a pop
-// at 200 vertices, against 1170 to 2000.  200 vertices, 1154 edges, weights to
-// 100: 193 -> 58 us with the read of the result (46 us the kernel); the 76
-// vertices left of RHG 2^20: 100 -> 40 us.  Eight neighbouring 16-bit columns a
-// lane, one load a pop, took 490 cycles: what it saves in loads it spends on
-// taking the columns apart and the popped vertex out.
-#include "mc_internal.cuh"
+// mc_dense.cu -- the launch of the dense rounds (mc_dense.cuh) on a graph in
+// device memory.
+#include "mc_dense.cuh"
 
 namespace mc {
 
 namespace {
 
+using DenseSmem = dense::DenseSmem<kDenseN>;
 constexpr int kN = kDenseN;
-constexpr int kThreads = 256;
-constexpr int kWarps = kThreads / 32;
-constexpr unsigned kAll = 0xffffffffu;
-constexpr int kSelf = -(1 << 30);  // on the diagonal: takes a vertex out as it is popped
-static_assert(kN == 224 && kThreads >= kN, "a lane owns seven columns at most, a thread one");
 
-struct DenseSmem {
-    int M[kN * kN];  // rows of kN
-    unsigned acc[kWarps][kN];
-    int par[kThreads], deg[kN], lab[kThreads], joinx[kN], first[kThreads + 1], cursor[kThreads], r[kN];
-    unsigned short perm[kN], orig[kThreads], order[kN];
-    u32 best[kWarps];
-    int wsum[kWarps];
-    i64 lam;
-    int un, len, arg;
-};
-
-__device__ __forceinline__ int sm_find(int *par, int x) {
-    volatile int *p = par;
-    while (true) {
-        const int q = p[x];
-        if (q == x) return x;
-        x = q;
-    }
-}
-
-__device__ __forceinline__ bool sm_union(int *par, int a, int b) {
-    while (true) {
-        a = sm_find(par, a);
-        b = sm_find(par, b);
-        if (a == b) return false;
-        if (a > b) {
-            const int t = a;
-            a = b;
-            b = t;
-        }
-        if (atomicCAS(&par[b], b, a) == b) return true;
-    }
-}
-
-// exclusive scan of one flag a thread; *total = the sum (all threads call)
-__device__ __forceinline__ int block_rank(bool flag, int *wsum, int *total) {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const unsigned m = __ballot_sync(kAll, flag);
-    if (lane == 0) wsum[wid] = __popc(m);
-    __syncthreads();
-    int before = 0, sum = 0;
-#pragma unroll
-    for (int w = 0; w < kWarps; ++w) {
-        before += w < wid ? wsum[w] : 0;
-        sum += wsum[w];
-    }
-    *total = sum;
-    __syncthreads();
-    return before + __popc(m & ((1u << lane) - 1u));
-}
-
-// the minimum degree below s.lam, if there is one, becomes the bound, with the
-// smallest such vertex as its side (n0 = vertices of the input)
-__device__ void take_min_degree(DenseSmem &s, int n, int n0) {
-    const int tid = threadIdx.x, lane = tid & 31;
-    if (tid < 32) {
-        int d = INT_MAX, arg = 0;
-        for (int v = lane; v < n; v += 32)
-            if (s.deg[v] < d) {
-                d = s.deg[v];
-                arg = v;
-            }
-        const int md = (int)__reduce_min_sync(kAll, (unsigned)d);
-        arg = (int)__reduce_min_sync(kAll, d == md ? (unsigned)arg : kAll);
-        if (lane == 0) {
-            s.arg = md < s.lam ? arg : -1;
-            if (md < s.lam) s.lam = md;
-        }
-    }
-    __syncthreads();
-    if (s.arg >= 0) {
-        const unsigned m = __ballot_sync(kAll, tid < n0 && s.orig[tid] == s.arg);
-        if (lane == 0) s.best[tid >> 5] = m;
-    }
-    __syncthreads();
-}
-
-// One capped scan (Alg. 3) by warp 0; a lane owns columns lane, lane + 32, ..,
-// KC of them.  A queue entry is min(r, C) << 8 | 255 - v: a vertex not reached
-// (r = 0) stays below 256, one popped (r far below 0, its key -1) below 0, and
-// no update needs to know which it was.  The next pop depends on the updates
-// alone; alpha and the joins follow while the maximum is on its way.
-template <int KC>
-__device__ void dense_scan(DenseSmem &s, int n, int start) {
-    const int lane = threadIdx.x;
-    const int C = (int)s.lam;
-    int r[KC], jx[KC];
-#pragma unroll
-    for (int k = 0; k < KC; ++k) {
-        r[k] = 0;
-        jx[k] = -1;
-        s.r[32 * k + lane] = 0;
-        s.order[32 * k + lane] = 0xffff;
-    }
-    __syncwarp();
-    i64 L = C, alpha = 0;
-    int Lj = C, nS = 0, len = 0, p = start;
-    while (true) {
-        int c[KC], e[KC];
-#pragma unroll
-        for (int k = 0; k < KC; ++k) c[k] = s.M[p * kN + 32 * k + lane];
-        const int dp = s.deg[p], rx = s.r[p];
-        __syncwarp();
-#pragma unroll
-        for (int k = 0; k < KC; ++k) {
-            r[k] += c[k];
-            s.r[32 * k + lane] = r[k];
-            const int key = r[k] < C ? (r[k] > -1 ? r[k] : -1) : C;
-            e[k] = key * 256 + (255 - 32 * k - lane);
-        }
-#pragma unroll
-        for (int o = 1; o < KC; o *= 2)
-#pragma unroll
-            for (int k = 0; k + o < KC; k += 2 * o) e[k] = e[k] > e[k + o] ? e[k] : e[k + o];
-        const int top = __reduce_max_sync(kAll, e[0]);
-        if (lane == 0) s.order[p] = (unsigned short)nS;
-        ++nS;
-        alpha += dp - 2LL * rx;
-        if (alpha < L && nS < n) {
-            L = alpha;
-            Lj = (int)alpha;
-            len = nS;
-        }
-#pragma unroll
-        for (int k = 0; k < KC; ++k)
-            if (r[k] >= Lj && r[k] - c[k] < Lj) jx[k] = p;
-        if (top < 256) break;
-        p = 255 - (top & 255);
-    }
-#pragma unroll
-    for (int k = 0; k < KC; ++k) s.joinx[32 * k + lane] = jx[k];
-    if (lane == 0) {
-        s.len = L < C ? len : 0;
-        s.lam = L;
-    }
-}
-
-__device__ __forceinline__ void dense_scan(DenseSmem &s, int n, int start) {
-    switch ((n + 31) / 32) {
-        case 1: return dense_scan<1>(s, n, start);
-        case 2: return dense_scan<2>(s, n, start);
-        case 3: return dense_scan<3>(s, n, start);
-        case 4: return dense_scan<4>(s, n, start);
-        case 5: return dense_scan<5>(s, n, start);
-        case 6: return dense_scan<6>(s, n, start);
-        default: return dense_scan<7>(s, n, start);
-    }
-}
-
-__global__ void __launch_bounds__(kThreads) k_dense(DevGraph g, i64 lam0, u64 seed, int pr_level, Status *out, u32 *bits_out) {
+__global__ void __launch_bounds__(dense::kThreads)
+k_dense(DevGraph g, i64 lam0, u64 seed, int pr_level, Status *out, u32 *bits_out) {
     extern __shared__ __align__(16) unsigned char raw[];
     DenseSmem &s = *reinterpret_cast<DenseSmem *>(raw);
     int *M = s.M;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int n0 = g.n;
-    int n = n0, err = 0;
     if (tid == 0) s.lam = lam0;
-    for (int i = tid; i < n0 * kN / 4; i += kThreads) reinterpret_cast<int4 *>(M)[i] = make_int4(0, 0, 0, 0);
+    for (int i = tid; i < n0 * kN / 4; i += dense::kThreads) reinterpret_cast<int4 *>(M)[i] = make_int4(0, 0, 0, 0);
     for (int i = lane; i < kN; i += 32) s.acc[wid][i] = 0;
     if (tid < kN) s.deg[tid] = 0;
     s.orig[tid] = (unsigned short)tid;
     __syncthreads();
-    for (int i = tid; i < (int)g.arcs; i += kThreads) {
+    for (int i = tid; i < (int)g.arcs; i += dense::kThreads) {
         const int2 e = g.adj[i];
         const int u = g.src[i], c = e.y < (int)lam0 ? e.y : (int)lam0;
         M[u * kN + e.x] = c;
         atomicAdd(&s.deg[u], c);
     }
-    if (tid < n0) M[tid * kN + tid] = kSelf;
+    if (tid < n0) M[tid * kN + tid] = dense::kSelf;
     __syncthreads();
-    int round = 0, guard = 0;
-    while (n >= 2 && s.lam > 0) {
-        if (++guard > 4 * n0 + 16) { err = MC_EINTERNAL; break; }
-        const i64 lam = s.lam;
-        s.par[tid] = tid;
-        if (tid == 0) s.un = 0;
-        __syncthreads();
-        // PR1/PR2 and the degree-2 rule, a warp a row (warp 0 scans meanwhile)
-        int un = 0;
-        if (pr_level >= 1 && wid > 0) {
-            for (int u = wid - 1; u < n; u += kWarps - 1) {
-                const int du = s.deg[u];
-                int cnt = 0, va = 0, vb = 0;  // the first two neighbours
-                for (int v0 = 0; v0 < n; v0 += 32) {
-                    const int v = v0 + lane;
-                    const int c = v < n ? M[u * kN + v] : 0;
-                    if (c > 0 && v > u) {
-                        const int dv = s.deg[v];
-                        if (c >= lam || (pr_level >= 2 && 2 * c > (du < dv ? du : dv))) un += sm_union(s.par, u, v);
-                    }
-                    unsigned m = __ballot_sync(kAll, c > 0);
-                    while (m && cnt < 3) {
-                        const int x = v0 + __ffs(m) - 1;
-                        m &= m - 1u;
-                        if (cnt == 0) va = x;
-                        if (cnt == 1) vb = x;
-                        ++cnt;
-                    }
-                }
-                if (pr_level >= 2 && cnt == 2 && lane == 0 && M[u * kN + va] == M[u * kN + vb])
-                    un += sm_union(s.par, u, va);
-            }
-        }
-        // one scan; its joins
-        if (wid == 0) {
-            const u64 h = splitmix64(seed ^ splitmix64((0x7A11ULL << 20) ^ (u64)round));
-            dense_scan(s, n, (int)(h % (u64)n));
-        }
-        __syncthreads();
-        if (tid < n && s.joinx[tid] >= 0) un += sm_union(s.par, s.joinx[tid], tid);
-        if (un) atomicAdd(&s.un, un);
-        __syncthreads();
-        ++round;
-        if (s.lam < lam) {
-            const int len = s.len;
-            const unsigned m = __ballot_sync(kAll, tid < n0 && s.order[s.orig[tid < n0 ? tid : 0]] < len);
-            if (lane == 0) s.best[wid] = m;
-            if (s.un == 0) {
-                __syncthreads();
-                continue;
-            }
-        }
-        if (s.un == 0) { err = MC_EINTERNAL; break; }
-        // number the blocks by their smallest members; the members in block order
-        const int root = tid < n ? sm_find(s.par, tid) : -1;
-        int nc = 0;
-        const int rank = block_rank(root == tid, s.wsum, &nc);
-        if (root == tid) s.lab[tid] = rank;
-        s.cursor[tid] = 0;
-        __syncthreads();
-        const int mine = tid < n ? s.lab[root] : 0;
-        __syncthreads();
-        if (tid < n) {
-            s.lab[tid] = mine;
-            atomicAdd(&s.cursor[mine], 1);
-        }
-        __syncthreads();
-        if (wid == 0) {
-            int carry = 0;
-            for (int b0 = 0; b0 < kThreads; b0 += 32) {
-                const int v = s.cursor[b0 + lane];
-                int inc = v;
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const int t = __shfl_up_sync(kAll, inc, o);
-                    if (lane >= o) inc += t;
-                }
-                s.first[b0 + lane] = carry + inc - v;
-                s.cursor[b0 + lane] = carry + inc - v;
-                carry += __shfl_sync(kAll, inc, 31);
-            }
-            if (lane == 0) s.first[kThreads] = carry;
-        }
-        __syncthreads();
-        if (tid < n) s.perm[atomicAdd(&s.cursor[mine], 1)] = (unsigned short)tid;
-        __syncthreads();
-        // rows: block a's members lie at a or later, so its sum may take row a
-        const int cap = (int)s.lam;
-        if (tid < n) {
-            for (int a = 0; a < nc; ++a) {
-                int sum = 0;
-                for (int i = s.first[a]; i < s.first[a + 1]; ++i) sum += M[s.perm[i] * kN + tid];
-                M[a * kN + tid] = sum < cap ? sum : cap;
-            }
-        }
-        __syncthreads();
-        // columns, and the degrees
-        unsigned *acc = s.acc[wid];
-        for (int a = wid; a < nc; a += kWarps) {
-            for (int v = lane; v < n; v += 32) {
-                const int c = M[a * kN + v], b = s.lab[v];
-                if (c > 0 && b != a) atomicAdd(&acc[b], (unsigned)c);
-            }
-            __syncwarp();
-            int d = 0;
-            for (int b = lane; b < n; b += 32) {
-                const unsigned x = acc[b];
-                const int c = x < (unsigned)cap ? (int)x : cap;
-                acc[b] = 0;
-                M[a * kN + b] = b == a ? kSelf : c;
-                d += c;
-            }
-            d = (int)__reduce_add_sync(kAll, (unsigned)d);
-            if (lane == 0) s.deg[a] = d;
-            __syncwarp();
-        }
-        if (tid < n0) s.orig[tid] = (unsigned short)s.lab[s.orig[tid]];
-        n = nc;
-        __syncthreads();
-        if (n >= 2) take_min_degree(s, n, n0);
-    }
-    __syncthreads();
+    const int err = dense::rounds(s, n0, seed, pr_level);
     if (s.lam < lam0 && tid < (n0 + 31) / 32) bits_out[tid] = s.best[tid];
     if (tid == 0) {
         out->lam = s.lam;
@@ -334,7 +42,7 @@ __global__ void __launch_bounds__(kThreads) k_dense(DevGraph g, i64 lam0, u64 se
 
 int dense_solve(const DevGraph &g, i64 lam, u64 seed, int pr_level, Status *out, u32 *bits_out, cudaStream_t s) {
     MC_CUDA(cudaFuncSetAttribute(k_dense, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(DenseSmem)));
-    ++::mc::g_launches; k_dense<<<1, kThreads, sizeof(DenseSmem), s>>>(g, lam, seed, pr_level, out, bits_out);
+    ++::mc::g_launches; k_dense<<<1, dense::kThreads, sizeof(DenseSmem), s>>>(g, lam, seed, pr_level, out, bits_out);
     MC_CUDA(cudaGetLastError());
     return MC_OK;
 }
