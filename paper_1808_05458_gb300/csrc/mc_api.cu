@@ -635,14 +635,33 @@ int solve_impl(mc_graph *g, const mc_options &o, cudaStream_t s, SolveOut &out) 
         }
         ph.mark(&S.ms_capforest);
         // contraction; the orig map and the new minimum degree ride on its
-        // final status read
+        // final status read.  Few enough blocks stop at the weights between
+        // them: the dense rounds add those up, the minimum degree included
+        Pairs few;
+        const bool few_ok = tail_n >= kDenseN && !cfg.pq_fifo && lam <= kDenseMaxLam;
         MC_TRY(contract_graph(cur, *nxt, w, lam, true, 0, s, [&]() -> int {
             MC_TRY(orig_update(w, n0, s));
             return min_degree(*nxt, w, s);
-        }, one_block));
+        }, one_block, few_ok ? &few : nullptr));
         if (w.h_st->err & kErrOverflow) return MC_EOVERFLOW;
         if (w.h_st->err & kErrNoProgress) return MC_EINTERNAL;
         bytes += cur.arcs * 20 + w.last_emitted * 12 + (i64)cur.n * 16 + (i64)n0 * 8;
+        if (few.n) {
+            ph.mark(&S.ms_contract);
+            ++rounds;
+            long long lt = lam;
+            if (few.n >= 2) {
+                MC_TRY(orig_update(w, n0, s));
+                MC_TRY(tail_solve_pairs(few, w, &lt, o.seed ^ (u64)rounds, o.pr_level, n0, s));
+                ph.mark(&S.ms_tail);
+                ++S.tail_launches;
+            }
+            if (verbose)
+                fprintf(stderr, "[mc]   contract -> n=%d emitted=%lld, tail lam %lld -> %lld (%.3f ms)\n", few.n,
+                        (long long)few.m, (long long)lam, lt, ph.last_ms());
+            lam = lt;
+            break;
+        }
         if (nxt->n >= 2 && w.h_st->mindeg < lam) {
             lam = w.h_st->mindeg;
             MC_TRY(side_from_vertex(w, n0, w.h_st->argmin, s));

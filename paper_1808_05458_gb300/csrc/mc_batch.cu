@@ -1668,6 +1668,30 @@ constexpr int kTailSmemN = 256;
 constexpr int kTailSmemArcs = 4096;
 constexpr int kTailSmemSN = 256;
 
+static int tail_room(Work &w, size_t need, cudaStream_t s) {
+    if (w.tail && w.tail_bytes >= need) return MC_OK;
+    dev_free(w.tail, s);
+    w.tail = nullptr;
+    w.tail_bytes = 0;
+    MC_TRY(dev_alloc(reinterpret_cast<void **>(&w.tail), need, s));
+    w.tail_bytes = need;
+    return MC_OK;
+}
+
+// the bound a tail launch left in the status and its side into lam and w
+static int tail_result(Work &w, const u32 *bits, int n0, long long *lam, cudaStream_t s) {
+    MC_TRY(status_read(w, s));
+    if (w.h_st->err) {
+        set_error_detail("tail solver failed");
+        return (int)w.h_st->err;
+    }
+    if (w.h_st->lam < *lam) {
+        MC_TRY(side_from_bits(w, n0, bits, s));
+        *lam = w.h_st->lam;
+    }
+    return MC_OK;
+}
+
 int tail_solve(const DevGraph &g, Work &w, int limit, long long *lam, u64 seed, int pr_level, int fifo,
                int n0, cudaStream_t s) {
     if (limit > 4096) limit = 4096;
@@ -1677,13 +1701,7 @@ int tail_solve(const DevGraph &g, Work &w, int limit, long long *lam, u64 seed, 
     const Layout L = on_chip ? make_layout(kTailSmemN, kTailSmemArcs) : make_layout(limit, 64LL * limit);
     // the side bitmap is read back from global memory in both cases
     const size_t need = on_chip ? al(4 * ((size_t)kTailSmemN / 32 + 2)) : L.bytes;
-    if (w.tail_bytes < need || !w.tail) {
-        dev_free(w.tail, s);
-        w.tail = nullptr;
-        w.tail_bytes = 0;
-        MC_TRY(dev_alloc(reinterpret_cast<void **>(&w.tail), need, s));
-        w.tail_bytes = need;
-    }
+    MC_TRY(tail_room(w, need, s));
     TailIn T;
     T.g = g;
     T.lam = *lam;
@@ -1708,18 +1726,15 @@ int tail_solve(const DevGraph &g, Work &w, int limit, long long *lam, u64 seed, 
         ++::mc::g_launches; k_tail<kTailSN, false><<<1, 32, 0, s>>>(T);
     }
     MC_CUDA(cudaGetLastError());
-    MC_TRY(status_read(w, s));
-    if (w.h_st->err) {
-        set_error_detail("tail solver failed");
-        return w.h_st->err;
-    }
-    if (w.h_st->lam < *lam) {
-        const u32 *bits = on_chip ? reinterpret_cast<const u32 *>(w.tail)
-                                  : reinterpret_cast<const u32 *>(w.tail + L.best);
-        MC_TRY(side_from_bits(w, n0, bits, s));
-        *lam = w.h_st->lam;
-    }
-    return MC_OK;
+    return tail_result(w, on_chip ? T.bits_out : reinterpret_cast<const u32 *>(w.tail + L.best), n0, lam, s);
+}
+
+int tail_solve_pairs(const Pairs &p, Work &w, long long *lam, u64 seed, int pr_level, int n0, cudaStream_t s) {
+    if (p.n < 2 || p.n > kDenseN || *lam > kDenseMaxLam) return MC_EINVAL;
+    MC_TRY(tail_room(w, al(4 * ((size_t)kTailSmemN / 32 + 2)), s));
+    u32 *bits = reinterpret_cast<u32 *>(w.tail);
+    MC_TRY(dense_solve_pairs(p, *lam, seed, pr_level, w.st, bits, s));
+    return tail_result(w, bits, n0, lam, s);
 }
 
 int batch_shapes() { return (int)(sizeof(kShapes) / sizeof(kShapes[0])); }

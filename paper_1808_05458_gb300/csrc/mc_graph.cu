@@ -741,7 +741,7 @@ static int build_from_pairs(i64 m, int nc, i64 clamp, int wb, DevGraph &out, Wor
 }
 
 int contract_graph(const DevGraph &in, DevGraph &out, Work &w, i64 clamp, bool flatten, int nc,
-                   cudaStream_t s, const std::function<int()> &post, bool one_block) {
+                   cudaStream_t s, const std::function<int()> &post, bool one_block, Pairs *pairs) {
     const int n = in.n;
     // count2 (the emitted arcs) starts at 0: zeroed by the flatten, else here
     if (!flatten) { ++::mc::g_launches; k_zero_count<<<1, 1, 0, s>>>(w.st); }
@@ -781,6 +781,11 @@ int contract_graph(const DevGraph &in, DevGraph &out, Work &w, i64 clamp, bool f
     const i64 m = w.h_st->count2;
     w.last_emitted = m;
     out.sym = in.sym;
+    // few enough blocks and pairs for the dense rounds: left as they are
+    if (pairs && in.sym && nc <= kDenseN && dense_takes_pairs(m, cap)) {
+        *pairs = Pairs{w.keysA, w.valsA, m, pack, nc};
+        return MC_OK;
+    }
     return build_from_pairs(m, nc, clamp, pack, out, w, s, post);
 }
 

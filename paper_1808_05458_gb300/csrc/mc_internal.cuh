@@ -178,6 +178,15 @@ void graph_free(DevGraph &g, cudaStream_t s);
 // read the status block back (synchronises the stream)
 int status_read(Work &w, cudaStream_t s);
 
+// the pairs of blocks a contraction emitted, n blocks (n = 0: they went into a
+// graph as usual)
+struct Pairs {
+    const u64 *keys = nullptr;
+    const int *vals = nullptr;
+    i64 m = 0;
+    int wb = 0, n = 0;
+};
+
 // ---------------------------------------------------------- path steps --
 // Sec. 2.1 contraction of `in` by union-find blocks in w.par (roots are the
 // smallest member): writes `out`, its degrees, lambda-hat update candidates
@@ -188,7 +197,8 @@ int status_read(Work &w, cudaStream_t s);
 // whose Status copy the caller may then use; w.last_emitted = arcs emitted.
 // With `one_block` the block of st->giant holds most vertices of `in`.
 int contract_graph(const DevGraph &in, DevGraph &out, Work &w, i64 clamp, bool flatten, int nc,
-                   cudaStream_t s, const std::function<int()> &post = {}, bool one_block = false);
+                   cudaStream_t s, const std::function<int()> &post = {}, bool one_block = false,
+                   Pairs *pairs = nullptr);
 
 // canonicalise raw CSR arrays (device) into `out` (drops self-loops / zero
 // weights, sums parallel arcs, sorts rows); checks symmetry if asked.
@@ -300,6 +310,11 @@ int tail_solve(const DevGraph &g, Work &w, int limit, long long *lam, u64 seed, 
 constexpr int kDenseN = 224;
 constexpr i64 kDenseMaxLam = (1 << 22) - 1;  // a column adds up below 2^30, a key's entry below 2^31
 int dense_solve(const DevGraph &g, i64 lam, u64 seed, int pr_level, Status *out, u32 *bits_out, cudaStream_t s);
+// the same on a contraction's emitted pairs, whose minimum degree it takes first
+constexpr i64 kDensePairs = 1 << 15;  // one block reads them: 128 a thread
+bool dense_takes_pairs(i64 m, i64 cap);  // m of them, weights to cap: their sums stay below 2^31
+int dense_solve_pairs(const Pairs &p, i64 lam, u64 seed, int pr_level, Status *out, u32 *bits_out, cudaStream_t s);
+int tail_solve_pairs(const Pairs &p, Work &w, long long *lam, u64 seed, int pr_level, int n0, cudaStream_t s);
 int side_from_bits(Work &w, int n0, const u32 *bits, cudaStream_t s);  // bit v = bits[orig[v]]
 void batch_set_shape(int shape);
 int batch_get_shape();
