@@ -52,7 +52,7 @@ using Dense = dense::DenseSmem<kDN>;
 struct CtaSmem {
     u32 best[kCtaMaxN / 32];
     int wsum[32];
-    int un, md, arg, graph;
+    int un, md, arg, graph, cross;
     unsigned tot;
 };
 
@@ -297,16 +297,21 @@ __device__ bool cta_solve(const CtaBatch &B, int gi, CtaSmem &s, unsigned char *
             s.arg = INT_MAX;
             s.un = 0;
             s.tot = 0;
+            s.cross = 0;
         }
         __syncthreads();
+        int cross = 0;
 #pragma unroll 4
         for (int e = tid; e < E; e += TH) {
             const int a = lab[ua[e]], b = lab[va[e]], w = wa[e];
             if (a != b) {
+                ++cross;
                 atomicAdd(&deg[a], w);
                 atomicAdd(&deg[b], w);
             }
         }
+        cross = (int)__reduce_add_sync(kAll, (unsigned)cross);
+        if (lane == 0 && cross) atomicAdd(&s.cross, cross);
         __syncthreads();
         int d = INT_MAX;
         unsigned tot = 0;
@@ -334,7 +339,9 @@ __device__ bool cta_solve(const CtaBatch &B, int gi, CtaSmem &s, unsigned char *
         // forests: more the closer the bound is to the mean degree, as many as fit
         int T = room / nb + 1;
         if (T < kMinT && T < lam) return false;
-        const i64 want = (kShare * lam * nb + s.tot - 1) / s.tot;
+        // (and units of at most the mean weight: a weight below one counts nothing)
+        const i64 share = kShare * nb > 2 * s.cross ? kShare * nb : 2 * s.cross;
+        const i64 want = (share * lam + s.tot - 1) / s.tot;
         const int most = poor ? kManyT : want < 3 ? 3 : want < kMaxT ? (int)want : kMaxT;
         T = T < most ? T : most;
         T = lam < T ? (int)lam : T;

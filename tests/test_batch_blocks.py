@@ -122,3 +122,10 @@ def test_faulty_graphs_are_refused(mc, fault):
     with pytest.raises(Exception):
         _run(mc, [good, (rp, col, w), good])
     _check(mc, [good])
+
+
+@pytest.mark.parametrize("wmax", [1, 3])
+def test_dense_rows_of_small_weights(mc, wmax):
+    # mean degrees far above the bound: units stay at the weights' size
+    _check(mc, [_random(n, d, wmax, 13 * n + int(d)) for n in (120, 400) for d in (40.0, 60.0)]
+           + [_two_cliques(60, 1, 5), _complete(150, wmax, 6)])
