@@ -211,10 +211,10 @@ int mc_min_cut(mc_graph *g, const mc_options *opt, int64_t *lambda_out,
  * queue order, canonical graphs of up to 2048 vertices whose state fits in
  * shared memory are solved one block per graph, by rounds of forest packing
  * and a dense finish.  The others (a batch mostly of several hundred graphs of
- * 33 to 95 vertices among them), and all of them under a chosen shape, go to one launch with a warp per graph, graphs
- * taken largest first (Alg. 2 per graph with full capped scans, PR1/PR2 when
- * opt->pr_level >= 1 and the kernel shape in use runs them, and
- * in-warp contraction).  Self-loops and zero weights are dropped and
+ * 33 to 95 vertices among them), and all of them under a chosen shape, go to
+ * one launch with a warp per graph, graphs taken largest first (Alg. 2 per
+ * graph with full capped scans, PR1/PR2 when opt->pr_level >= 1 and the kernel
+ * shape in use runs them, and in-warp contraction).  Self-loops and zero weights are dropped and
  * parallel arcs merged; after that every graph must be symmetric (each arc
  * (u, v, c) has its mirror (v, u, c)), which the kernel checks per graph; a
  * disconnected graph gets lambda 0.  stats: n_input/m_input are totals,
@@ -234,8 +234,9 @@ int mc_batch_min_cut(int32_t G, const int64_t *vtx_off, const int64_t *arc_off,
  * mc_batch_autotune -- time every batched-kernel shape (warps per block x
  * vertices whose scan state fits in shared memory per warp x whether the
  * in-warp PR1/PR2 tests run, which never changes a lambda) on this batch,
- * keep the fastest for later mc_batch_min_cut calls on the current device
- * of this process, and report it.  Arguments as mc_batch_min_cut;
+ * keep the fastest (or the default, where that is faster than all of them)
+ * for later mc_batch_min_cut calls on the current device of this process, and
+ * report the fastest shape.  Arguments as mc_batch_min_cut;
  * ms_per_shape (max_shapes entries, may be NULL) receives each shape's
  * kernel time.  The shapes' results are not returned.
  */

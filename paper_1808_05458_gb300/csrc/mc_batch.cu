@@ -1489,7 +1489,7 @@ int batch_solve(int G, const long long *vtx_off, const long long *arc_off, const
         return arc_off[x + 1] - arc_off[x] > arc_off[y + 1] - arc_off[y];
     });
 
-    if (shape < 0) shape = g_shape_choice;
+    if (shape == -1) shape = g_shape_choice;
     const bool tuned = shape >= 0;
     if (!tuned) shape = default_shape(G, nmax);
     // a batch nobody tuned goes to the block-per-graph solver first, and what

@@ -294,7 +294,9 @@ size_t full_block_words(int n, int cap);
 int flatten_raw(int *par, int *root, int *cnt, int n, cudaStream_t s);
 
 // many graphs, one warp per graph (layout of mc_batch_min_cut, host arrays);
-// shape < 0 = the tuned or default configuration; *ms_out = kernel time
+// shape -1 = the tuned or default configuration, kBatchDefaultShape = the
+// default whatever was chosen; *ms_out = kernel time
+constexpr int kBatchDefaultShape = -2;
 int batch_solve(int G, const long long *vtx_off, const long long *arc_off, const int *row_ptr,
                 const int *col, const int *w, const mc_options &o, long long *lambdas, u32 *bitmaps,
                 const long long *bitmap_word_off, int shape, double *ms_out);
