@@ -364,28 +364,44 @@ def run_gpu(args, rank, world, local_rank):
     h2d = sum(a.nbytes for a in host)
     d2h = 8 + 4 * ((n + 31) // 32)
 
-    # dominant kernel: the concurrent CAPFOREST scan kernel
+    # the dominant part of the step: the concurrent CAPFOREST scans where a round
+    # ran them, else the first round's certificates without scans
     scan_ms = sum(s["ms_scan_kernel"] for s in stats)
     scan_launches = sum(s["scan_launches"] for s in stats)
     scanned_arcs = sum(s["scanned_arcs"] for s in stats)
     scanned_verts = sum(s["scanned_verts"] for s in stats)
-    # per scanned arc: 8 B {neighbour, weight}; per scanned vertex: 8 B row
-    # offsets + 8 B degree + 4 B owner claim + 4 B visit order
-    alg_bytes = scanned_arcs * 8 + scanned_verts * 24
-    per_launch_bytes = alg_bytes / max(1, scan_launches)
-    per_launch_s = scan_ms / max(1, scan_launches) / 1000.0
+    pr_ms = sum(s["ms_pr"] for s in stats)
+    forest_ms = sum(s["ms_capforest"] for s in stats)
+    bound0 = stats[-1]["bound_initial"]
     peak, peak_kind = measured_peaks()
+    tr = None
+    if scan_launches and scan_ms >= max(pr_ms, forest_ms - scan_ms):
+        name = "k_capforest (concurrent capped CAPFOREST scans)"
+        # per scanned arc: 8 B {neighbour, weight}; per scanned vertex: 8 B row
+        # offsets + 8 B degree + 4 B owner claim + 4 B visit order
+        part_ms, launches, alg_bytes = scan_ms, scan_launches, scanned_arcs * 8 + scanned_verts * 24
+        tr = kernel_traffic("k_capforest")
+    elif pr_ms >= forest_ms:
+        name = "triangle tests of the first round (k_tri_first, k_tri_collect, k_tri_jobs, k_par_flatten)"
+        # per vertex: 64 B of offsets, labels and first arcs for each of three
+        # tests, and about `bound` common neighbours of 8 B in the two rows of each
+        part_ms, launches, alg_bytes = pr_ms, args.steps, args.steps * n * (48 * bound0 + 192)
+    else:
+        name = "forest packing of the first round (k_pack_start .. k_pack_fill)"
+        # per vertex: `bound` parents of 4 B written and read (and their arcs), 16 B of offsets
+        part_ms, launches, alg_bytes = forest_ms, args.steps, args.steps * n * (20 * bound0 + 16)
+    per_launch_bytes = alg_bytes / max(1, launches)
+    per_launch_s = part_ms / max(1, launches) / 1000.0
     achieved = per_launch_bytes / per_launch_s / 1e9 if per_launch_s > 0 else 0.0
-    tr = kernel_traffic("k_capforest")
-    roofline = {"kernel": "k_capforest (concurrent capped CAPFOREST scans)", "bound": "hbm",
+    roofline = {"kernel": name, "bound": "hbm",
                 "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                 "peak_source": f"{peak_kind} hbm_gbs",
-                # one capture on RHG n=2^19 round 0, scaled by algorithmic bytes
+                # for the scans, one capture on RHG n=2^19 round 0, scaled by algorithmic bytes
                 "traffic": tr["traffic_over_alg"] * per_launch_bytes if tr else None,
                 "traffic_source": "profiles/k_capforest_rhg2e19.md" if tr else None,
                 "alg_bytes_per_launch": per_launch_bytes,
                 "ms_per_launch": per_launch_s * 1000.0,
-                "share_of_step": scan_ms / max(1e-9, total_ms)}
+                "share_of_step": part_ms / max(1e-9, total_ms)}
 
     cpu = None
     if rank == 0 and world == 1 and not args.no_cpu:
