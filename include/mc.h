@@ -218,7 +218,8 @@ int mc_min_cut(mc_graph *g, const mc_options *opt, int64_t *lambda_out,
  * parallel arcs merged; after that every graph must be symmetric (each arc
  * (u, v, c) has its mirror (v, u, c)), which the kernel checks per graph; a
  * disconnected graph gets lambda 0.  stats: n_input/m_input are totals,
- * ms_total is the kernels' device time.
+ * ms_total is the kernels' device time, from the first launch to the last one's
+ * end (a large batch's arcs are still arriving meanwhile).
  * Errors: MC_EINVAL (n_g < 2, bad offsets -- a graph's first offset not 0 or
  * its last not its arc count, refused before any launch, or an offset below
  * its predecessor, found by the kernel before it reads that graph's arcs --,

@@ -514,11 +514,11 @@ int batch_cta_class(int n, long long m) {
 
 bool batch_cta_chain(int n) { return n > kFew && n < kCtaChainN; }
 
-int batch_cta_launch(const CtaBatch &B, cudaStream_t s) {
+int batch_cta_launch(const CtaBatch &B, const cudaStream_t (&s)[kCtaClasses]) {
     static_assert(kCtaClasses == 3, "");
-    MC_TRY(launch_class<0>(B, s));
-    MC_TRY(launch_class<1>(B, s));
-    return launch_class<2>(B, s);
+    MC_TRY(launch_class<0>(B, s[0]));
+    MC_TRY(launch_class<1>(B, s[1]));
+    return launch_class<2>(B, s[2]);
 }
 
 }  // namespace mc

@@ -30,6 +30,7 @@ struct CtaBatch {
 int batch_cta_class(int n, long long m);
 // graphs the matrix's one chain may take longer for than the packing
 bool batch_cta_chain(int n);
-int batch_cta_launch(const CtaBatch &B, cudaStream_t s);
+// a launch for each class that has graphs, on its stream
+int batch_cta_launch(const CtaBatch &B, const cudaStream_t (&s)[kCtaClasses]);
 
 }  // namespace mc

@@ -129,3 +129,24 @@ def test_dense_rows_of_small_weights(mc, wmax):
     # mean degrees far above the bound: units stay at the weights' size
     _check(mc, [_random(n, d, wmax, 13 * n + int(d)) for n in (120, 400) for d in (40.0, 60.0)]
            + [_two_cliques(60, 1, 5), _complete(150, wmax, 6)])
+
+
+def test_large_batch_in_chunks(mc):
+    # more arcs than a batch that is copied whole; graphs for the warps among
+    # them, and a fault in the last chunk
+    kinds = [_random(n, d, 50, 17 * n) for n, d in ((1500, 6.0), (2000, 5.0), (50, 8.0), (700, 12.0), (2100, 4.0))]
+    kinds.append(graphgen.random_connected(300, 1500, seed=3, wmax=9))
+    want = [oracle.noi(*g)[0] for g in kinds]
+    order = np.random.default_rng(1).integers(0, len(kinds), 6000)
+    gs = [kinds[k] for k in order]
+    assert sum(len(g[1]) for g in gs) >= 32 << 20
+    for _ in range(2):
+        lam, sides = _run(mc, gs)
+        assert lam.tolist() == [want[k] for k in order]
+        for j in range(0, len(gs), 241):
+            assert oracle.cut_weight(*gs[j], sides[j]) == lam[j]
+    rp, col, w = (x.copy() for x in kinds[0])
+    w[5] += 1
+    with pytest.raises(Exception):
+        _run(mc, gs + [(rp, col, w)])
+    assert _run(mc, gs)[0].tolist() == [want[k] for k in order]
