@@ -194,7 +194,7 @@ def run_reference(args, rank, world):
 def form_batched(mc, peak, seed=1):
     """The batched form (4096 graphs, n in 50..2000, degree 4..16, weights
     1..100): one mc_batch_min_cut per step through the C ABI from pinned host
-    arrays (H2D of the batch, one persistent launch, D2H of the lambdas and
+    arrays (H2D of the batch, the solvers' launches, D2H of the lambdas and
     side bitmaps), every lambda checked against the oracle's lambdas stored
     in tests/golden/batch_lambdas_seed1.json (written by the script beside
     it), and the plain path (mc_graph_create + mc_min_cut per graph) timed on
@@ -256,7 +256,7 @@ def form_batched(mc, peak, seed=1):
         "lambda_checked": f"all {G} equal to the oracle's stored NOI results",
         "roofline": {"bound": "hbm", "achieved": alg / kern / 1e9, "peak": peak, "unit": "GB/s",
                      "frac": alg / kern / 1e9 / peak, "traffic": None,
-                     "note": "one warp per graph; latency-bound (dependent per-pop loads)"},
+                     "note": "a block per graph (a warp for the rest); bound by the packing's walks in shared memory"},
     }
 
 
