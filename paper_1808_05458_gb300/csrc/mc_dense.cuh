@@ -150,6 +150,7 @@ __device__ inline void dense_scan(DenseSmem<N> &s, int n, int start) {
             const int key = r[k] < C ? (r[k] > -1 ? r[k] : -1) : C;
             e[k] = key * 256 + (255 - 32 * k - lane);
         }
+        __syncwarp();  // the next pop's r comes from another lane's store
 #pragma unroll
         for (int o = 1; o < KC; o *= 2)
 #pragma unroll
