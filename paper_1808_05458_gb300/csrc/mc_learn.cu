@@ -914,10 +914,17 @@ struct Proposer {
     u64 feat_seed = 0x51ED270B27A4BB1DULL;
 };
 
+// (an allocation that fails leaves none of the old pointers behind: the next
+// call, or the release, would use memory that is somebody else's by then)
 static int prop_alloc(Proposer &p, int n, cudaStream_t s) {
     if (n <= p.n_cap) return MC_OK;
-    void *ps[] = {p.X, p.Z, p.S, p.dH, p.dG, p.rd, p.fd, p.Hb, p.Gb, p.dZb, p.Sm0, p.Sm1};
-    for (void *q : ps) dev_free(q, s);
+    p.n_cap = 0;
+    auto drop = [&](auto *&q) {
+        dev_free(q, s);
+        q = nullptr;
+    };
+    drop(p.X), drop(p.Z), drop(p.S), drop(p.dH), drop(p.dG), drop(p.rd), drop(p.fd);
+    drop(p.Hb), drop(p.Gb), drop(p.dZb), drop(p.Sm0), drop(p.Sm1);
     const size_t N = (size_t)n;
     MC_TRY(dev_alloc_n(&p.Sm0, N, s));
     MC_TRY(dev_alloc_n(&p.Sm1, N, s));
