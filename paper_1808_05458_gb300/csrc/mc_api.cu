@@ -515,6 +515,8 @@ int solve_impl(mc_graph *g, const mc_options &o, cudaStream_t s, SolveOut &out) 
                                g->two_arc_rows0 == 0;
         if (o.pr_level > 0 && !pr12_idle) {
             MC_TRY(pr_tests_budget(cur, w, thr, 1, o.pr_level < 2 ? o.pr_level : 2, 64, s));
+            // (the unions that follow walk over what these left)
+            if (cur.n > kMeet) MC_TRY(flatten_parents(w, cur.n, s));
             bytes += cur.arcs * 16;
         }
         ph.mark(&S.ms_pr);

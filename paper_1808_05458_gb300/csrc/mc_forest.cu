@@ -35,6 +35,8 @@
 //
 // Bound by L2 latency and random sectors: per unit of weight 8 bytes of arcs,
 // one store and about eight loads of parents.
+#include <algorithm>
+
 #include "mc_internal.cuh"
 
 namespace mc {
@@ -61,8 +63,7 @@ struct Pack {
 
 __device__ __forceinline__ bool owns(int u, i64 du, int v, i64 dv) { return du < dv || (du == dv && u > v); }
 
-__device__ __forceinline__ bool apart(const int *p, int a, int b) { return root_of(p, a) != root_of(p, b); }
-
+// the 32-bit mixer "lowbias32" of C. Wellons' published hash search (2018)
 __device__ __forceinline__ unsigned mix32(unsigned x) {
     x ^= x >> 16;
     x *= 0x7feb352du;
@@ -169,14 +170,18 @@ __global__ void __launch_bounds__(kThreads) k_pack_start_wide(const DevGraph g, 
 
 // every vertex points at its root; forest after forest, so that the parents
 // walked over stay in L2
-__global__ void __launch_bounds__(kThreads) k_pack_flatten(Pack P) {
+__global__ void __launch_bounds__(kFlatThreads, kFlatBlocks) k_pack_flatten(Pack P) {
     const unsigned total = (unsigned)P.n * (unsigned)P.t, stride = gridDim.x * blockDim.x;
-    for (unsigned k = blockIdx.x * blockDim.x + threadIdx.x; k < total; k += stride) {
-        int *p = P.F + k / (unsigned)P.n * (unsigned)P.n;
-        const int u = (int)(k % (unsigned)P.n);
-        const int p0 = ld_parent(p + u), r = root_of(p, p0);
-        if (r != p0) p[u] = r;
-    }
+    flatten_rounds([&](auto fresh) {
+        bool any = false;
+        for (unsigned k = blockIdx.x * blockDim.x + threadIdx.x; k < total; k += stride) {
+            int *p = P.F + k / (unsigned)P.n * (unsigned)P.n;
+            const int u = (int)(k % (unsigned)P.n);
+            const int p0 = ld_parent(p + u), r = root_near<fresh.value>(p, p0, &any);
+            if (r != p0) p[u] = r;
+        }
+        return any;
+    });
 }
 
 // One union a vertex and forest, for every `every`-th 32 vertices of a forest
@@ -203,10 +208,10 @@ __global__ void __launch_bounds__(kThreads) k_pack_join(const DevGraph g, Pack P
             if (!owns(u, du, v, g.deg[v])) continue;
         }
         int *p = P.F + j * (unsigned)P.n;
-        if (!apart(p, u, v)) continue;
+        if (uf_meet<false>(p, u, v) != 1) continue;
         const u32 bit = 1u << (i & 31);
         if (atomicOr(&P.taken[i >> 5], bit) & bit) continue;  // another forest has it
-        if (!uf_join(p, u, v)) atomicAnd(&P.taken[i >> 5], ~bit);
+        if (uf_meet<true>(p, u, v) != 1) atomicAnd(&P.taken[i >> 5], ~bit);
     }
 }
 
@@ -338,13 +343,14 @@ k_pack_fill(const DevGraph g, Pack P, int *par, const int *__restrict__ reps, in
             int nm = 0;
             for (int j0 = 0; j0 < P.t; j0 += 32) {
                 const int j = j0 + lane;
-                const bool off = j < P.t && apart(P.F + j * P.n, u, rr[(k - 1) * P.t + j]);
+                const bool off = j < P.t && uf_meet<false>(P.F + j * P.n, u, rr[(k - 1) * P.t + j]) != 0;
                 const unsigned m = __ballot_sync(0xffffffffu, off);
                 if (off) miss[nm + __popc(m & ((1u << lane) - 1u))] = (unsigned short)j;
                 nm += __popc(m);
             }
             __syncwarp();
             int got = 0;
+            bool lost = false;  // a walk that was cut off united nothing
             for (int i0 = first; i0 < a1 && got < nm; i0 += 32) {
                 const int i = i0 + lane;
                 int c = 0, v = u;
@@ -372,11 +378,11 @@ k_pack_fill(const DevGraph g, Pack P, int *par, const int *__restrict__ reps, in
                     }
                 }
                 const int inc = warp_incl_sum(c), s = got + inc - c;
-                for (int x = s; x < s + c && x < nm; ++x) uf_join(P.F + miss[x] * P.n, u, v);
+                for (int x = s; x < s + c && x < nm; ++x) lost |= uf_meet<true>(P.F + miss[x] * P.n, u, v) < 0;
                 got += __shfl_sync(0xffffffffu, inc, 31);
             }
             __syncwarp();
-            if (got >= nm && lane == 0) {
+            if (!__any_sync(0xffffffffu, lost) && got >= nm && lane == 0) {
                 un += uf_union(par, u, reps[k - 1]);
                 __threadfence();  // its unions are out before it counts as in the block
                 *(volatile int *)&in[u] = k;
@@ -414,11 +420,12 @@ int forest_round(const DevGraph &g, Work &w, i64 t, cudaStream_t s) {
     ++::mc::g_launches;
     if (g.n < kWideN) k_pack_start_wide<<<blocks_for((i64)g.n * 32), kThreads, 0, s>>>(g, P);
     else k_pack_start<<<blocks_for(g.n), kThreads, 0, s>>>(g, P);
-    ++::mc::g_launches; k_pack_flatten<<<blocks_for(words), kThreads, 0, s>>>(P);
+    const int flat = std::min(blocks_for(words), num_sms() * kFlatBlocks);
+    ++::mc::g_launches; k_pack_flatten<<<flat, kFlatThreads, 0, s>>>(P);
     i64 every = g.arcs / words;
     every = every < 1 ? 1 : (every > 16 ? 16 : every);
     ++::mc::g_launches; k_pack_join<<<blocks_for(words / every + 32 * t), kThreads, 0, s>>>(g, P, (unsigned)every);
-    ++::mc::g_launches; k_pack_flatten<<<blocks_for(words), kThreads, 0, s>>>(P);
+    ++::mc::g_launches; k_pack_flatten<<<flat, kFlatThreads, 0, s>>>(P);
     ++::mc::g_launches; k_pack_reps<<<1, kSample * kParts, 0, s>>>(P, reps, &w.st->giant);
     const size_t smem = sizeof(int) * kReps * (size_t)t;  // at most 32 KB
     ++::mc::g_launches; k_pack_blocks<<<blocks_for((i64)g.n * 8), kThreads, smem, s>>>(P, w.par, reps, w.T, w.st);

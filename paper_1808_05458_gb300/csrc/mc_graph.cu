@@ -94,18 +94,52 @@ int union_find_init(int *par, int n, cudaStream_t s) {
     return MC_OK;
 }
 
-// flatten: root[v] = root of v in par; cnt[v] = (v is a root).  par is not
-// written here, so the walks read it through the read-only cache (measured
-// against path-halving finds on RHG 2^20: solve 1.79 -> 1.72 ms); the roots
-// go to their own array.
-__global__ void k_flatten(const int *__restrict__ par, int *__restrict__ root, int *__restrict__ cnt, int n, Status *st) {
+// flatten: root[v] = root of v in par; cnt[v] = (v is a root).  The walks read
+// through L1 and write no parent where they are short (measured against
+// path-halving finds on RHG 2^20: solve 1.79 -> 1.72 ms); the roots go to their
+// own array.
+__global__ void __launch_bounds__(kFlatThreads, kFlatBlocks)
+k_flatten(int *par, int *__restrict__ root, int *__restrict__ cnt, int n, Status *st) {
     if (st && blockIdx.x == 0 && threadIdx.x == 0) st->count2 = 0;  // the emit counter
-    for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
-        int r = v, p = __ldg(par + v);
-        while (p != r) { r = p; p = __ldg(par + r); }
-        cnt[v] = (r == v);
-        root[v] = r;
-    }
+    flatten_rounds([&](auto fresh) {
+        bool any = false;
+        for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
+            bool cut = false;
+            const int r = root_near<fresh.value>(par, v, &cut);
+            if (cut) par[v] = r;
+            any |= cut;
+            cnt[v] = (r == v);
+            root[v] = r;
+        }
+        return any;
+    });
+}
+
+// every vertex points at its root
+__global__ void __launch_bounds__(kFlatThreads, kFlatBlocks) k_par_flatten(int *par, int n) {
+    flatten_rounds([&](auto fresh) {
+        bool any = false;
+        for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
+            const int p = ld_parent(par + v), r = root_near<fresh.value>(par, p, &any);
+            if (r != p) par[v] = r;
+        }
+        return any;
+    });
+}
+
+static int flat_grid(int n) {
+    const int b = (n + kFlatThreads - 1) / kFlatThreads, most = num_sms() * kFlatBlocks;
+    return b < most ? b : most;
+}
+
+static void launch_flatten(int *par, int *root, int *cnt, int n, Status *st, cudaStream_t s) {
+    ++::mc::g_launches; k_flatten<<<flat_grid(n), kFlatThreads, 0, s>>>(par, root, cnt, n, st);
+}
+
+int flatten_parents(Work &w, int n, cudaStream_t s) {
+    ++::mc::g_launches; k_par_flatten<<<flat_grid(n), kFlatThreads, 0, s>>>(w.par, n);
+    MC_CUDA(cudaGetLastError());
+    return MC_OK;
 }
 
 // lab[v] = lab[root(v)]; roots already hold their new id from the scan
@@ -747,7 +781,7 @@ int contract_graph(const DevGraph &in, DevGraph &out, Work &w, i64 clamp, bool f
     if (!flatten) { ++::mc::g_launches; k_zero_count<<<1, 1, 0, s>>>(w.st); }
     const int *d_nc = nullptr;
     if (flatten) {
-        ++::mc::g_launches; k_flatten<<<grid_for(n), kThreads, 0, s>>>(w.par, w.root, w.cnt, n, w.st);
+        launch_flatten(w.par, w.root, w.cnt, n, w.st, s);
         d_nc = reinterpret_cast<int *>(&w.st->count);
         MC_TRY(exclusive_scan_i32(w.cnt, w.lab, n, reinterpret_cast<int *>(&w.st->count), w.scan_tmp, &w.st->err, s));
         ++::mc::g_launches; k_relabel<<<grid_for(n), kThreads, 0, s>>>(w.root, w.lab, n);
@@ -1030,11 +1064,11 @@ int connected_components(const DevGraph &g, Work &w, int *ncomp, cudaStream_t s)
     if (g.arcs > 0) {
         int *giant = reinterpret_cast<int *>(&w.st->count2);
         ++::mc::g_launches; k_cc_sample<<<grid_for((i64)g.n * kCcSample), kThreads, 0, s>>>(g, w.par);
-        ++::mc::g_launches; k_flatten<<<grid_for(g.n), kThreads, 0, s>>>(w.par, w.root, w.cnt, g.n, nullptr);
+        launch_flatten(w.par, w.root, w.cnt, g.n, nullptr, s);
         ++::mc::g_launches; k_cc_giant<<<1, kCcProbe, 0, s>>>(w.root, g.n, giant);
         ++::mc::g_launches; k_cc_finish<<<grid_for((i64)g.n * 32), kThreads, 0, s>>>(g, w.root, giant, w.par);
     }
-    ++::mc::g_launches; k_flatten<<<grid_for(g.n), kThreads, 0, s>>>(w.par, w.root, w.cnt, g.n, nullptr);
+    launch_flatten(w.par, w.root, w.cnt, g.n, nullptr, s);
     ++::mc::g_launches; k_zero_count<<<1, 1, 0, s>>>(w.st);
     MC_TRY(exclusive_scan_i32(w.cnt, w.lab, g.n, reinterpret_cast<int *>(&w.st->count), w.scan_tmp, &w.st->err, s));
     MC_TRY(status_read(w, s));
@@ -1110,7 +1144,7 @@ int orig_update(Work &w, int n0, cudaStream_t s) {
 namespace mc {
 
 int flatten_labels(Work &w, int n, cudaStream_t s) {
-    ++::mc::g_launches; k_flatten<<<grid_for(n), kThreads, 0, s>>>(w.par, w.root, w.cnt, n, nullptr);
+    launch_flatten(w.par, w.root, w.cnt, n, nullptr, s);
     MC_CUDA(cudaGetLastError());
     return MC_OK;
 }
@@ -1206,7 +1240,7 @@ int iota_i32(int *a, int n, cudaStream_t s) {
 
 // flatten a caller-provided union-find array: root[v] = root of v
 int flatten_raw(int *par, int *root, int *cnt, int n, cudaStream_t s) {
-    ++::mc::g_launches; k_flatten<<<grid_for(n), kThreads, 0, s>>>(par, root, cnt, n, nullptr);
+    launch_flatten(par, root, cnt, n, nullptr, s);
     MC_CUDA(cudaGetLastError());
     return MC_OK;
 }

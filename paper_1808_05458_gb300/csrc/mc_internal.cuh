@@ -269,6 +269,7 @@ int pr_triangles(const DevGraph &g, Work &w, i64 lam, bool unit, cudaStream_t s)
 // st->giant, their share (of 256) -> st->giant_share; w.root from a flatten
 int find_giant(Work &w, int n, cudaStream_t s);
 int flatten_labels(Work &w, int n, cudaStream_t s);   // w.root[v] = root of v in w.par
+int flatten_parents(Work &w, int n, cudaStream_t s);  // w.par[v] = root of v
 int round_reset(Work &w, i64 lam, cudaStream_t s);    // st->lam = lam, counters = 0
 int round_start(Work &w, int n, i64 lam, cudaStream_t s);  // union_find_init + round_reset
 int side_canon(Work &w, int n0, cudaStream_t s);
@@ -379,6 +380,53 @@ __device__ __forceinline__ int ld_parent(const int *p) {
     return v;
 }
 
+// Parents a walk goes over before it leaves the one it came to as its own: on a
+// graph numbered along a path the unions of one kernel, each right by itself,
+// leave chains as long as the graph, and walks to the root would take n loads
+// that wait for one another.  (A path of 2^20 vertices: 0.9 ms the whole solve;
+// 378 ms with walks that halve the chain as uf_find does, the walkers meeting at
+// the same few words, 587 ms with the halving by compare and swap; flattening in
+// three launches, the later two mostly with nothing to do, cost the small graphs
+// 20 us a solve.)
+constexpr int kWalk = 64;
+
+__device__ __forceinline__ int ld_parent_l2(const int *p) {
+    int v;
+    asm volatile("ld.global.cg.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+
+// the root above x, or the ancestor kWalk parents up (*far)
+template <bool FRESH>
+__device__ __forceinline__ int root_near(const int *p, int x, bool *far) {
+    for (int k = 0; k < kWalk; ++k) {
+        const int q = FRESH ? ld_parent_l2(p + x) : ld_parent(p + x);
+        if (q == x) return x;
+        x = q;
+    }
+    *far = true;
+    return x;
+}
+
+// Flattens parents in rounds.  `round` walks up from all vertices of this thread
+// (root_near), leaves what a walk that was cut off came to as the vertex's parent,
+// and says whether there were any.  A thread writes its own vertices' parents
+// alone, so that a round of all threads divides what is left of every chain by
+// kWalk; the first reads through L1, the others what the rounds before wrote.  On
+// grids of the resident threads at most: what lies above is not shortened before
+// its thread begins.
+constexpr int kFlatThreads = 256, kFlatBlocks = 8;  // a SM
+template <bool V>
+struct Fresh {
+    static constexpr bool value = V;
+};
+template <class F>
+__device__ __forceinline__ void flatten_rounds(F round) {
+    bool more = round(Fresh<false>());
+    while (more) more = round(Fresh<true>());
+}
+
+// the root above x in parents that are flat
 __device__ __forceinline__ int root_of(const int *p, int x) {
     while (true) {
         const int q = ld_parent(p + x);
@@ -387,24 +435,39 @@ __device__ __forceinline__ int root_of(const int *p, int x) {
     }
 }
 
-// links the larger root to the smaller one; false if the ends were connected.
-// What was read may be old: a root that is none any more fails its CAS (which
-// returns its parent as it is), and a node that was a root has a smaller root
-// now, so no cycle closes.
-__device__ __forceinline__ bool uf_join(int *p, int a, int b) {
-    a = root_of(p, a);
-    b = root_of(p, b);
-    while (a != b) {
-        if (a < b) {
-            const int t = a;
+// Both ends walk up, the one with the larger parent first, until they meet or
+// that one is a root: parents are smaller than their children (in a forest,
+// past the first, whose parents are roots by then), so the ends are apart, and
+// UNITE links the root below the other's parent.  On a chain that is a few steps
+// where the ends are near each other, whatever its length.  1: apart (and
+// united); 0: together; -1: neither after `most` parents.  What is read may be
+// old: a root that is none any more fails its CAS (which returns its parent as
+// it is), and an ancestor stays one.
+constexpr int kMeet = 1024;
+template <bool UNITE>
+__device__ __forceinline__ int uf_meet(int *p, int a, int b, int most = kMeet) {
+    int pa = ld_parent(p + a), pb = ld_parent(p + b);
+    for (int k = 0; k < most; ++k) {
+        if (pa == pb) return 0;
+        if (pa < pb) {
+            int t = a;
             a = b;
             b = t;
+            t = pa;
+            pa = pb;
+            pb = t;
         }
-        const int old = atomicCAS(p + a, a, b);
-        if (old == a) return true;
-        a = root_of(p, old);
+        if (pa == a) {
+            if (!UNITE) return 1;
+            const int old = atomicCAS(p + a, a, pb);
+            if (old == a) return 1;
+            pa = old;
+            continue;
+        }
+        a = pa;
+        pa = ld_parent(p + a);
     }
-    return false;
+    return -1;
 }
 
 // as uf_union; *root = the root of the merged set (its smallest member)

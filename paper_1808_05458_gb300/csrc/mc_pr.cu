@@ -49,7 +49,7 @@ __global__ void k_pr(const DevGraph g, int *par, long long lam, int lo, int leve
         const long long du = g.deg[u], dv = g.deg[v];
         bool ok = (lo <= 1 && level >= 1 && c >= lam) ||
                   (lo <= 2 && level >= 2 && 2 * c > (du < dv ? du : dv));
-        if (ok && uf_union(par, u, v)) ++local;
+        if (ok && uf_meet<true>(par, u, v, INT_MAX) > 0) ++local;
     }
     // degree-2 tie rule: a vertex with exactly two neighbours of equal weight
     // joins the smaller one (a cut below delta slides along such a path)
@@ -58,7 +58,7 @@ __global__ void k_pr(const DevGraph g, int *par, long long lam, int lo, int leve
             const int a = g.rp[u];
             if (g.rp[u + 1] - a != 2) continue;
             const int2 e0 = g.adj[a], e1 = g.adj[a + 1];
-            if (e0.y == e1.y && uf_union(par, u, e0.x < e1.x ? e0.x : e1.x)) ++local;
+            if (e0.y == e1.y && uf_meet<true>(par, u, e0.x < e1.x ? e0.x : e1.x, INT_MAX) > 0) ++local;
         }
     }
     if (local) atomicAdd(unions, (unsigned long long)local);
@@ -133,7 +133,7 @@ k_pr34(const DevGraph g, int *par, long long lam, int lo, int level, int budget,
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) pr4 += __shfl_xor_sync(0xffffffffu, pr4, o);
                 const bool ok = __any_sync(0xffffffffu, pr3) || (level >= 4 && cc + pr4 >= lam);
-                if (ok && lane == 0 && uf_union(par, u, vv)) ++local;
+                if (ok && lane == 0 && uf_meet<true>(par, u, vv, INT_MAX) > 0) ++local;
             }
         }
     }
@@ -223,7 +223,7 @@ k_pr34_pairs(const DevGraph g, int *par, long long lam, int lo, int level, int m
         __syncwarp();
         for (int j = lane; j < ne; j += 32) {
             const bool ok = sm.pr3[j] != 0 || (level >= 4 && (long long)sm.cv[j] + (long long)sm.pr4[j] >= lam);
-            if (ok && uf_union(par, u, sm.v[j])) ++local;
+            if (ok && uf_meet<true>(par, u, sm.v[j], INT_MAX) > 0) ++local;
         }
         __syncwarp();
     }
@@ -335,19 +335,11 @@ k_tri_first(const DevGraph g, int *par, int need, int max_steps, unsigned long l
         const int sum = tri_test<UNIT>(g, t, need, max_steps);
         if (t.u >= 0 && sum >= need && (threadIdx.x & 7) == 0) {
             if (t.v < u && atomicCAS(&par[u], u, t.v) == u) ++local;
-            else local += uf_join(par, u, t.v);
+            else local += uf_meet<true>(par, u, t.v) > 0;
         }
         __syncwarp();
     }
     tri_count(local, unions);
-}
-
-// every vertex points at its root
-__global__ void k_par_flatten(int *par, int n) {
-    for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
-        const int p = ld_parent(par + v), r = root_of(par, p);
-        if (r != p) par[v] = r;
-    }
 }
 
 // the jobs of the next pass: of each vertex the first of its first eight arcs
@@ -415,33 +407,33 @@ k_tri_jobs(const DevGraph g, int *par, const u64 *__restrict__ jobs, const u64 *
             t = TriJob{(int)(job >> 32), e.x, e.y};
         }
         const int sum = tri_test<UNIT>(g, t, need, max_steps);
-        if (t.u >= 0 && sum >= need && (threadIdx.x & 7) == 0) local += uf_join(par, t.u, t.v);
+        if (t.u >= 0 && sum >= need && (threadIdx.x & 7) == 0) local += uf_meet<true>(par, t.u, t.v) > 0;
         __syncwarp();
     }
     tri_count(local, unions);
 }
 
 template <bool UNIT>
-static void launch_triangles(const DevGraph &g, Work &w, int need, cudaStream_t s) {
+static int launch_triangles(const DevGraph &g, Work &w, int need, cudaStream_t s) {
     const int max_steps = 16 + (need < 4096 ? need : 4096);
     auto *un = reinterpret_cast<unsigned long long *>(&w.st->unions);
     u64 *count = reinterpret_cast<u64 *>(&w.st->count), *jobs = w.keysA;
-    int fb = (g.n + 255) / 256, jb = (int)(((i64)g.n * 8 + 255) / 256);
+    int jb = (int)(((i64)g.n * 8 + 255) / 256);
     if (jb > num_sms() * 8) jb = num_sms() * 8;
     ++::mc::g_launches; k_tri_first<UNIT><<<jb, 256, 0, s>>>(g, w.par, need, max_steps, un);
-    if (fb > num_sms() * 8) fb = num_sms() * 8;
     for (int pass = 0; pass < 2; ++pass) {
-        ++::mc::g_launches; k_par_flatten<<<fb, 256, 0, s>>>(w.par, g.n);
-        cudaMemsetAsync(count, 0, sizeof(u64), s);
+        MC_TRY(flatten_parents(w, g.n, s));
+        MC_CUDA(cudaMemsetAsync(count, 0, sizeof(u64), s));
         ++::mc::g_launches; k_tri_collect<<<(int)(((i64)g.n * 2 + 255) / 256), 256, 0, s>>>(g, w.par, pass ? 8 : 2, jobs, count);
         ++::mc::g_launches; k_tri_jobs<UNIT><<<jb, 256, 0, s>>>(g, w.par, jobs, count, need, max_steps, un);
     }
+    return MC_OK;
 }
 
 int pr_triangles(const DevGraph &g, Work &w, i64 lam, bool unit, cudaStream_t s) {
     if (lam >= kTriMaxBound || g.arcs == 0) return MC_OK;
-    if (unit) launch_triangles<true>(g, w, (int)lam, s);
-    else launch_triangles<false>(g, w, (int)lam, s);
+    if (unit) MC_TRY(launch_triangles<true>(g, w, (int)lam, s));
+    else MC_TRY(launch_triangles<false>(g, w, (int)lam, s));
     MC_CUDA(cudaGetLastError());
     return MC_OK;
 }
