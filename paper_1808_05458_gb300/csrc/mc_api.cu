@@ -218,6 +218,7 @@ int create_impl(int32_t n, const int32_t *row_ptr, const int32_t *col, const int
     }
     g->device_ptrs = dev;
     g->n0 = n;
+    g->w.own = A > n ? A : n;
     cudaStream_t s = g->stream;
     const int *drp = row_ptr, *dcol = col, *dw = w;
     // host input: the raw arrays are staged in Ga (rp, src) and Gb (src);

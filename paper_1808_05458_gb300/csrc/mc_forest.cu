@@ -400,11 +400,12 @@ int blocks_for(i64 threads) {
 
 }  // namespace
 
-// the forests lie in the contraction's key buffer (2 ints an arc of the input)
+// The forests lie in the contraction's key buffer, 2 ints an arc of the input.
+// Only what this input needs of it counts: a buffer kept from a larger graph
+// holds more, and the rounds a graph goes through must not depend on that.
 bool forest_fits(const DevGraph &g, const Work &w, i64 t) {
     const i64 words = t * (i64)g.n;
-    return t >= 1 && t <= kForestMaxT && words <= 2 * (w.cap_arcs > w.cap_n ? w.cap_arcs : w.cap_n) &&
-           words < kInt32Max;
+    return t >= 1 && t <= kForestMaxT && words <= 2 * w.own && words < kInt32Max;
 }
 
 int forest_round(const DevGraph &g, Work &w, i64 t, cudaStream_t s) {

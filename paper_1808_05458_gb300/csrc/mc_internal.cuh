@@ -161,6 +161,7 @@ struct Work {
     Status *st = nullptr;
     Status *h_st = nullptr;  // pinned mirror
     i64 cap_n = 0, cap_arcs = 0;
+    i64 own = 0;             // what the key buffers hold in a graph made for this input alone
     i64 last_emitted = 0;    // arcs emitted by the last contraction
     // single-warp tail solver scratch (allocated on first use)
     unsigned char *tail = nullptr;
