@@ -478,6 +478,7 @@ int solve_impl(mc_graph *g, const mc_options &o, cudaStream_t s, SolveOut &out) 
     // thr has found a real cut, which lowers lam as well.
     auto exact_loop = [&](DevGraph cur, DevGraph *nxt) -> int {
     int guard = 0;
+    int pack_n = INT_MAX;  // forest packing on graphs of at most so many vertices
     i64 delta_cur = g->delta0;
     if (o.approx_milli > 0 && cur.rp != g->G0.rp && cur.n >= 2) {
         MC_TRY(min_degree(cur, w, s));
@@ -560,7 +561,13 @@ int solve_impl(mc_graph *g, const mc_options &o, cudaStream_t s, SolveOut &out) 
         // 762 K vertices an RHG graph's first contraction left, the forests
         // united four in five, the scans thirteen in fourteen).  A round that
         // unites less than an eighth of the vertices has the scans try as well.
-        bool packed = false, one_block = false;
+        // After a packing that did, the next waits until half of the vertices are
+        // gone: on a grid it then unites all of them, but on graphs that shrink by
+        // a few vertices a round it never does (random 8-regular graphs of 16384
+        // vertices with weights to 100, about 90 rounds: 44 to 56 ms with a packing in
+        // every round, 32 to 41 so; 1024 x 1024 grid: 2.0 ms both ways, 2.5 with none
+        // after the first).
+        bool packed = false, one_block = false, tried = true;
         const bool input = cur.rp == g->G0.rp;
         if (quick && g->clustered && input && o.pr_level >= 4 && thr < kTriMaxBound) {
             MC_TRY(pr_triangles(cur, w, thr, g->wmax0 == 1, s));
@@ -579,11 +586,14 @@ int solve_impl(mc_graph *g, const mc_options &o, cudaStream_t s, SolveOut &out) 
             MC_TRY(status_read(w, s));
             unions = w.h_st->unions;
             packed = unions * 8 >= cur.n;
+            if (!packed) pack_n = cur.n / 2;
             one_block = unions * 2 >= cur.n;
             // heads of the rows, and each parent written once and read twice
             bytes += (i64)cur.n * thr * 20 + (i64)cur.n * 16;
+        } else {
+            tried = false;
         }
-        if (verbose && quick)
+        if (verbose && tried)
             fprintf(stderr, "[mc] round %d n=%d arcs=%lld lam=%lld: unions=%lld without scans\n", rounds, cur.n,
                     (long long)cur.arcs, (long long)thr, (long long)unions);
         // reading the rows outside the largest block pays where there is much
