@@ -581,7 +581,7 @@ int solve_impl(mc_graph *g, const mc_options &o, cudaStream_t s, SolveOut &out) 
             // common neighbours in each of three tests' two rows
             bytes += (i64)cur.n * (3 * 16 * thr + 3 * 64);
             ph.mark(&S.ms_pr);
-        } else if (quick && (!g->clustered || (!input && cur.n < (1 << 17))) && forest_fits(cur, w, thr)) {
+        } else if (quick && cur.n <= pack_n && (!g->clustered || (!input && cur.n < (1 << 17))) && forest_fits(cur, w, thr)) {
             MC_TRY(forest_round(cur, w, thr, s));
             MC_TRY(status_read(w, s));
             unions = w.h_st->unions;
