@@ -1560,6 +1560,7 @@ int batch_solve(int G, const long long *vtx_off, const long long *arc_off, const
         return arc_off[x + 1] - arc_off[x] > arc_off[y + 1] - arc_off[y];
     });
 
+    const bool whole = shape == kBatchDefaultShape;  // timed against the shapes: kernels alone, as theirs
     if (shape == -1) shape = g_shape_choice;
     const bool tuned = shape >= 0;
     if (!tuned) shape = default_shape(G, nmax);
@@ -1584,7 +1585,7 @@ int batch_solve(int G, const long long *vtx_off, const long long *arc_off, const
     // the other leave idle.  A chunk costs its own last graphs' time, so that only
     // large batches gain: 42 M arcs 3.91 -> 3.16 ms a call (eight chunks 4.02), 21 M
     // 2.15 -> 2.21, 10 M 1.33 -> 1.79 (before the classes ran side by side).
-    const int chunks = cta && arc_off[G] >= kChunkArcs ? kChunks : 1;
+    const int chunks = cta && !whole && arc_off[G] >= kChunkArcs ? kChunks : 1;
     std::vector<int> split((size_t)chunks + 1, 0);  // graphs
     for (int q = 1; q <= chunks; ++q)
         split[q] = q == chunks ? G : (int)(std::lower_bound(arc_off, arc_off + G + 1, arc_off[G] / chunks * q) - arc_off);

@@ -297,7 +297,9 @@ int flatten_raw(int *par, int *root, int *cnt, int n, cudaStream_t s);
 
 // many graphs, one warp per graph (layout of mc_batch_min_cut, host arrays);
 // shape -1 = the tuned or default configuration, kBatchDefaultShape = the
-// default whatever was chosen; *ms_out = kernel time
+// default whatever was chosen, with the batch copied whole before the kernels
+// whatever its size; *ms_out = kernel time (in chunks: with the copies of all but
+// the first)
 constexpr int kBatchDefaultShape = -2;
 int batch_solve(int G, const long long *vtx_off, const long long *arc_off, const int *row_ptr,
                 const int *col, const int *w, const mc_options &o, long long *lambdas, u32 *bitmaps,
