@@ -1372,7 +1372,7 @@ __global__ void __launch_bounds__(32) k_tail(TailIn T) {
 
 // ------------------------------------------------------------ host side --
 constexpr int kChunks = 4;
-constexpr long long kChunkArcs = 32 << 20;
+constexpr long long kChunkArcs = 28 << 20;
 struct BatchCtx {
     unsigned char *scratch = nullptr;
     size_t scratch_bytes = 0;
@@ -1583,8 +1583,9 @@ int batch_solve(int G, const long long *vtx_off, const long long *arc_off, const
     // on one while the next is on its way: each chunk has its own lists and
     // launches, on two streams in turn so that one fills what the last graphs of
     // the other leave idle.  A chunk costs its own last graphs' time, so that only
-    // large batches gain: 42 M arcs 3.91 -> 3.16 ms a call (eight chunks 4.02), 21 M
-    // 2.15 -> 2.21, 10 M 1.33 -> 1.79 (before the classes ran side by side).
+    // large batches gain, from between 26 and 30 M (2^20) arcs on: 10.4 M 1.05 ms a
+    // call whole and 1.84 in chunks, 20.4 M 2.07 and 2.31, 25.7 M 2.40 and 2.58, 30.5 M
+    // 2.82 and 2.63, 40.4 M 3.88 and 3.25, 60.3 M 5.71 and 4.26.
     const int chunks = cta && !whole && arc_off[G] >= kChunkArcs ? kChunks : 1;
     std::vector<int> split((size_t)chunks + 1, 0);  // graphs
     for (int q = 1; q <= chunks; ++q)
