@@ -156,6 +156,47 @@ __device__ void cta_side(CtaSmem &s, int n, F f) {
     }
 }
 
+// The rule for degree 2 (mc_pr.cu) on the blocks: one with exactly two edges
+// out, of equal weight, goes with the end of one of them.  A packing unites two
+// vertices of a cycle a round, and a cycle given up went through the warps after
+// all: 300 cycles of 200 to 1100 vertices 3.2 ms a call, 0.21 so (2.8 by the warps
+// alone).  Returns the unions; x: 3 nb ints.
+template <int TH>
+__device__ int cta_paths(CtaSmem &s, const unsigned short *lab, const unsigned short *ua, const unsigned short *va,
+                         const unsigned short *wa, int E, int nb, unsigned short *par, int *x) {
+    int *cnt = x, *diff = x + nb, *pick = x + 2 * nb;
+    __syncthreads();  // s.un has been read
+    for (int b = threadIdx.x; b < nb; b += TH) {
+        cnt[b] = 0;
+        diff[b] = 0;
+        pick[b] = INT_MAX;
+    }
+    if (threadIdx.x == 0) s.un = 0;
+    __syncthreads();
+    for (int e = threadIdx.x; e < E; e += TH) {
+        const int a = lab[ua[e]], b = lab[va[e]], w = wa[e];
+        if (a == b) continue;
+        atomicAdd(&cnt[a], 1);
+        atomicAdd(&cnt[b], 1);
+        atomicXor(&diff[a], w);
+        atomicXor(&diff[b], w);
+        atomicMin(&pick[a], e);
+        atomicMin(&pick[b], e);
+    }
+    __syncthreads();
+    int un = 0;
+    for (int e = threadIdx.x; e < E; e += TH) {
+        const int a = lab[ua[e]], b = lab[va[e]];
+        if (a == b) continue;
+        const bool take = (cnt[a] == 2 && diff[a] == 0 && pick[a] == e) || (cnt[b] == 2 && diff[b] == 0 && pick[b] == e);
+        if (take && !meet16<true>(par, a, b)) ++un;
+    }
+    un = (int)__reduce_add_sync(kAll, (unsigned)un);
+    if ((threadIdx.x & 31) == 0 && un) atomicAdd(&s.un, un);
+    __syncthreads();
+    return s.un;
+}
+
 // one graph; false = left to the warp-per-graph solver.  All threads call, and
 // agree on what they return.
 template <int TH>
@@ -377,10 +418,10 @@ __device__ bool cta_solve(const CtaBatch &B, int gi, CtaSmem &s, unsigned char *
             if (!poor && T < kManyT && lam > T) {
                 poor = true;
                 if (united == 0) continue;
-            } else if (nb > kDN) {
-                return false;
-            } else {
+            } else if (nb <= kDN) {
                 break;
+            } else if (B.pr_level < 2 || cta_paths<TH>(s, lab, ua, va, wa, E, nb, par, reinterpret_cast<int *>(F)) * 8 < nb) {
+                return false;
             }
         }
         // number the blocks (in deg) by their smallest members
