@@ -383,9 +383,10 @@ def run_gpu(args, rank, world, local_rank):
         tr = kernel_traffic("k_capforest")
     elif pr_ms >= forest_ms:
         name = "triangle tests of the first round (k_tri_first, k_tri_collect, k_tri_jobs, k_par_flatten)"
-        # per vertex: 64 B of offsets, labels and first arcs for each of three
-        # tests, and about `bound` common neighbours of 8 B in the two rows of each
-        part_ms, launches, alg_bytes = pr_ms, args.steps, args.steps * n * (48 * bound0 + 192)
+        # at least: a test a vertex (two rows' offsets and about `bound` common
+        # neighbours of 8 B in each); what the second and third pass test, the
+        # vertices the first left, is not counted
+        part_ms, launches, alg_bytes = pr_ms, args.steps, args.steps * n * (16 * bound0 + 16)
     else:
         name = "forest packing of the first round (k_pack_start .. k_pack_fill)"
         # per vertex: `bound` parents of 4 B written and read (and their arcs), 16 B of offsets

@@ -369,7 +369,7 @@ int lp_bound(mc_graph *g, const mc_options &o, i64 &lam, cudaStream_t s, bool ve
             MC_TRY(orig_update(w, n0, s));
             return min_degree(*nxt, w, s);
         }));
-        bytes += cur.arcs * 20;
+        bytes += cur.arcs * 12;
         const i64 delta_cl = w.h_st->mindeg;
         if (delta_cl < lam) {
             lam = delta_cl;
@@ -453,7 +453,7 @@ int solve_impl(mc_graph *g, const mc_options &o, cudaStream_t s, SolveOut &out) 
     MC_TRY(iota_i32(w.orig, n0, s));
     i64 lam = g->delta0;
     MC_TRY(side_from_vertex(w, n0, g->argmin0, s));
-    bytes += g->G0.arcs * 8 + (i64)n0 * 12;  // degree sweep
+    bytes += (i64)n0 * 4;
 
     ScanConfig cfg;
     cfg.pq_fifo = o.pq_order == MC_PQ_FIFO;
@@ -577,9 +577,9 @@ int solve_impl(mc_graph *g, const mc_options &o, cudaStream_t s, SolveOut &out) 
             unions = w.h_st->unions;
             packed = unions * 8 >= cur.n;
             one_block = w.h_st->giant_share >= 192;
-            // offsets, labels and the first arcs of every row, and about `thr`
-            // common neighbours in each of three tests' two rows
-            bytes += (i64)cur.n * (3 * 16 * thr + 3 * 64);
+            // a test: two rows' offsets and about `thr` common neighbours in each;
+            // every vertex's first arc, and twice its offsets and label
+            bytes += ((i64)cur.n + w.h_st->tests) * (16 * thr + 16) + (i64)cur.n * 32;
             ph.mark(&S.ms_pr);
         } else if (quick && cur.n <= pack_n && (!g->clustered || (!input && cur.n < (1 << 17))) && forest_fits(cur, w, thr)) {
             MC_TRY(forest_round(cur, w, thr, s));
@@ -658,7 +658,10 @@ int solve_impl(mc_graph *g, const mc_options &o, cudaStream_t s, SolveOut &out) 
         }, one_block, few_ok ? &few : nullptr));
         if (w.h_st->err & kErrOverflow) return MC_EOVERFLOW;
         if (w.h_st->err & kErrNoProgress) return MC_EINTERNAL;
-        bytes += cur.arcs * 20 + w.last_emitted * 12 + (i64)cur.n * 16 + (i64)n0 * 8;
+        // an arc: source, neighbour and weight; of the rows outside one block at
+        // least the arcs that gave a pair
+        bytes += (one_block && cur.sym ? w.last_emitted * 4 : cur.arcs * 12) + w.last_emitted * 12 + (i64)cur.n * 16 +
+                 (i64)n0 * 8;
         if (few.n) {
             ph.mark(&S.ms_contract);
             ++rounds;
@@ -706,7 +709,7 @@ int solve_impl(mc_graph *g, const mc_options &o, cudaStream_t s, SolveOut &out) 
         // the LP bound's and is not taken here
         int nc = 0;
         MC_TRY(cluster_level0(g, o.lp_iters > 0 ? o.lp_iters : 2, o.seed ^ 0x9E37ULL, lam, &nc, s));
-        bytes += (g->G0.arcs * 12 + (i64)n0 * 12) * 2 * (o.lp_iters > 0 ? o.lp_iters : 2) + g->G0.arcs * 20;
+        bytes += (g->G0.arcs * 12 + (i64)n0 * 12) * 2 * (o.lp_iters > 0 ? o.lp_iters : 2) + g->G0.arcs * 12;
         if (nc >= 2) MC_TRY(proposer_on_clusters(g, *pp, g->Ga, w.h_st->mindeg, lam, verbose, s));
         MC_TRY(iota_i32(w.orig, n0, s));
     }

@@ -1188,6 +1188,7 @@ __device__ __forceinline__ void round_reset_body(Status *st, long long lam) {
     st->scanned_verts = 0;
     st->scans = 0;
     st->blacklisted = 0;
+    st->tests = 0;
     st->err = 0;
 }
 

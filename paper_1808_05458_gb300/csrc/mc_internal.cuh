@@ -99,6 +99,7 @@ struct Status {
     int giant;           // a vertex of the block most vertices are in (forest rounds)
     int giant_share;     // how many of the 256 vertices find_giant looks at are in it
     int wedges, closed;  // wedges probed and closed (graph creation)
+    i64 tests;           // triangle tests of the second and third pass
 };
 
 constexpr int kErrAsym = 1;       // asymmetric input

@@ -394,8 +394,9 @@ k_tri_collect(const DevGraph g, const int *__restrict__ par, int q1, u64 *jobs, 
 template <bool UNIT>
 __global__ void __launch_bounds__(256, 8)
 k_tri_jobs(const DevGraph g, int *par, const u64 *__restrict__ jobs, const u64 *count, int need, int max_steps,
-           unsigned long long *unions) {
+           unsigned long long *unions, i64 *tests) {
     const i64 nj = (i64)*count;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *tests += nj;
     const i64 step = (i64)gridDim.x * blockDim.x / 8;
     int local = 0;
     for (i64 k0 = ((i64)blockIdx.x * blockDim.x + (threadIdx.x & ~31)) / 8; k0 < nj; k0 += step) {
@@ -425,7 +426,7 @@ static int launch_triangles(const DevGraph &g, Work &w, int need, cudaStream_t s
         MC_TRY(flatten_parents(w, g.n, s));
         MC_CUDA(cudaMemsetAsync(count, 0, sizeof(u64), s));
         ++::mc::g_launches; k_tri_collect<<<(int)(((i64)g.n * 2 + 255) / 256), 256, 0, s>>>(g, w.par, pass ? 8 : 2, jobs, count);
-        ++::mc::g_launches; k_tri_jobs<UNIT><<<jb, 256, 0, s>>>(g, w.par, jobs, count, need, max_steps, un);
+        ++::mc::g_launches; k_tri_jobs<UNIT><<<jb, 256, 0, s>>>(g, w.par, jobs, count, need, max_steps, un, &w.st->tests);
     }
     return MC_OK;
 }
