@@ -68,19 +68,21 @@ __global__ void k_rand_init(DevGraph g, u64 seed, double2 *__restrict__ S, doubl
 }
 
 // One lazy random-walk step: out = (in + D^-1 A in) / 2 (a vertex without arcs
-// keeps in / 2).  Bound by the FP64 pipe, where a warp instruction takes 16
-// cycles of a SM whatever lanes it serves: eight lanes a vertex, so that a warp
-// reduces and finishes four vertices with the instructions of one (even lanes
-// the first sum, odd lanes the second), the reciprocals taken once before the
-// first step, and weights of 1 not converted.  A row of more than kLongRow
-// arcs gets the whole warp.  32768 vertices, 1 M arcs: 80 us a step with a warp
-// a vertex, 20 so (four lanes a vertex: 24).
+// keeps in / 2).  A step is one wave of warps, each waiting for three loads one
+// after another (offsets, arcs, the neighbours' values: 21 long-scoreboard stalls an
+// issue, 15 % of the issue slots used), and then for FP64 sums, where a warp
+// instruction takes 16 cycles of a SM whatever lanes it serves.  So eight lanes
+// a vertex, and a warp loads for, reduces and finishes four vertices with the
+// instructions of one (even lanes the first sum, odd lanes the second), the
+// reciprocals taken once before the first step, and weights of 1 not converted.
+// A row of more than kLongRow arcs gets the whole warp.  32768 vertices, 1 M arcs:
+// 80 us a step with a warp a vertex, 20 so (four lanes a vertex: 24).
 constexpr int kLongRow = 128;
 constexpr int kSmoothLg = 3;  // eight lanes a vertex
 
 __device__ __forceinline__ void smooth_arcs(const DevGraph &g, const double2 *__restrict__ in, int i, int i1, int step,
                                             double &sx, double &sy) {
-        constexpr int kU = 4;
+    constexpr int kU = 4;
     for (; __any_sync(0xffffffffu, i < i1); i += kU * step) {
         int2 e[kU];
         double2 x[kU];
