@@ -25,9 +25,9 @@
 // graphs, random graphs).  There the scans' regions meet before any certifies
 // much, and a round ended in the full scan, one pop after another.  Solve
 // times before and after: 50-core of an R-MAT graph of scale 18 (21 K
-// vertices, lambda-hat 99) 42.9 -> 0.36 ms, 10-core at scale 20 (247 K
-// vertices, 14.5 M edges, lambda-hat 12) 5.05 -> 0.27 ms, two joined random
-// blocks of 2048 vertices 3.13 -> 0.45 ms.  On clustered graphs (hyperbolic,
+// vertices, lambda-hat 99) 42.9 -> 0.26 ms, 10-core at scale 20 (247 K
+// vertices, 14.5 M edges, lambda-hat 12) 5.05 -> 0.23 ms, two joined random
+// blocks of 2048 vertices 3.13 -> 0.30 ms.  On clustered graphs (hyperbolic,
 // n = 2^20) the forests fall apart into stretches that differ from forest to
 // forest -- 0.4 % of the vertices united after 0.59 ms -- while the scans
 // unite 95 % in 0.75 ms; the solver tells the two apart by the share of closed
@@ -169,7 +169,8 @@ __global__ void __launch_bounds__(kThreads) k_pack_start_wide(const DevGraph g, 
 }
 
 // every vertex points at its root; forest after forest, so that the parents
-// walked over stay in L2
+// walked over stay in L2.  Bound by their latency (41 long-scoreboard stalls an
+// issue); 21 K vertices, t = 99: 15 and 11 us, 20 and 17 on four times the blocks.
 __global__ void __launch_bounds__(kFlatThreads, kFlatBlocks) k_pack_flatten(Pack P) {
     const unsigned total = (unsigned)P.n * (unsigned)P.t, stride = gridDim.x * blockDim.x;
     flatten_rounds([&](auto fresh) {
@@ -188,7 +189,8 @@ __global__ void __launch_bounds__(kFlatThreads, kFlatBlocks) k_pack_flatten(Pack
 // (another 32 in the next): an owned arc behind the row's head, if it connects
 // anything.  About weight / t of a vertex's units are spare, and a forest's
 // trees are fewer than a tenth of its vertices, so a share of the vertices
-// that falls as the rows grow joins nearly all of them.
+// that falls as the rows grow joins nearly all of them.  Bound by parents from
+// L2: 21 K vertices, t = 99, 31 us (52 with a walk to the root from each end).
 __global__ void __launch_bounds__(kThreads) k_pack_join(const DevGraph g, Pack P, unsigned every) {
     const unsigned m = ((P.n + 31u) / 32u + every - 1u) / every * 32u, total = m * (unsigned)P.t;
     const unsigned stride = gridDim.x * blockDim.x;
