@@ -31,7 +31,7 @@ struct mc_graph {
     int argmin0 = 0;
     i64 wmax0 = 0;          // largest arc weight of G0
     i64 two_arc_rows0 = 0;  // rows of G0 with exactly two arcs
-    bool clustered = false; // most wedges of G0 are closed (k_graph_stats)
+    bool clustered = false; // a third of the wedges of G0 are closed (k_graph_stats)
     bool device_ptrs = false;
     bool complete = false;  // every buffer allocated and the input built
     std::vector<cudaEvent_t> events;  // phase-clock events, reused across calls
@@ -291,7 +291,7 @@ int create_impl(int32_t n, const int32_t *row_ptr, const int32_t *col, const int
         g->argmin0 = g->w.h_st->argmin;
         g->wmax0 = g->w.h_st->count;
         g->two_arc_rows0 = g->w.h_st->count2;
-        g->clustered = 2 * g->w.h_st->closed > g->w.h_st->wedges;
+        g->clustered = 3 * g->w.h_st->closed > g->w.h_st->wedges;
         if (g->delta0 >= (1LL << 62)) rc = MC_EOVERFLOW;
     }
     if (rc != MC_OK) {

@@ -678,9 +678,14 @@ __global__ void k_zero_count(Status *st) {
 // row has two arcs, PR1, PR2 and the degree-2 rule cannot unite anything.
 // The first blocks also probe kWedges wedges (two arcs of an evenly spaced
 // vertex): st->closed of the st->wedges found have their ends adjacent.  Above
-// one half the graph is clustered (hyperbolic graphs 0.75-0.77; R-MAT cores
-// 0.11-0.26, random graphs below 0.14, at every size looked at), and its
-// rounds are the scans'; else the forest packing's (mc_forest.cu).
+// a third the graph is clustered and its first round is the triangle tests';
+// else the forest packing's (mc_forest.cu).  Hyperbolic graphs have 0.75-0.77,
+// triangulated grids 0.4, R-MAT cores from scale 16 on 0.16-0.26 up to the 50-core,
+// random graphs below 0.14.  In between (a line at one half against one at a
+// third): triangulated grid of 2^20 vertices 1.60 and 0.41 ms, of 2^14 0.73 and 0.18;
+// R-MAT scale 16 80-core (0.34) 28.6 and 0.70, scale 14 50-core (0.37) 4.1 and 0.54,
+// 30-core (0.33) 0.23 and 0.47; small worlds of 2^16 vertices, eight to a side and
+// 15 % rewired, 0.82 and 1.21, four and 10 % 1.03 and 0.48.
 constexpr int kWedges = 1024;
 
 __global__ void k_graph_stats(const DevGraph g, Status *st) {
